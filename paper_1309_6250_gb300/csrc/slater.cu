@@ -26,32 +26,15 @@
 // or in double-float (slater_cdf_kernel).
 #include <cmath>
 
-#include "eval_common.cuh"
+#include "slater_common.cuh"
 
 namespace qmcspl {
 namespace {
 
 constexpr int kSlaterThreads = 256;
-#ifndef QMCSPL_SLATER_DF_THREADS
-#define QMCSPL_SLATER_DF_THREADS 512
-#endif
 // double-float kernel: one CTA per SM (its matrix fills shared memory), so the CTA itself
 // must bring the warps that hide the latency of the dependent FP32 chains
-constexpr int kSlaterDfThreads = QMCSPL_SLATER_DF_THREADS;
-constexpr int kSlaterMaxBlock = QMCSPL_SLATER_MAX_BLOCK;
-
-struct SlaterArgs {
-    const void* val;
-    const void* grad;
-    const void* lap;
-    long long n_walkers;
-    int n_elec, n_up, n_orb;
-    double* logdet;
-    double* sign;
-    double* kinetic;
-    double* drift;
-    int arith;                // 0: FP64, 1: double-float
-};
+constexpr int kSlaterDfThreads = 512;
 
 template <typename T>
 __device__ __forceinline__ double ld(const void* p, long long i)
@@ -238,21 +221,12 @@ __global__ void __launch_bounds__(kSlaterThreads) slater_kernel(const SlaterArgs
     }
 }
 
-// 1 / d in double-float: one Newton step on the float reciprocal, e = 1 - d y to ~2^-48.
-__device__ __forceinline__ dfloat df_recip(dfloat d)
-{
-    const float y = 1.0f / d.h;
-    const float p = __fmul_rn(d.h, y);
-    const float pe = fmaf(d.h, y, -p);                  // d.h y = p + pe exactly
-    const float e = __fsub_rn(__fsub_rn(__fsub_rn(1.0f, p), pe), __fmul_rn(d.l, y));
-    return df_norm(y, __fmul_rn(y, e));
-}
-
-// The same computation in double-float.  Shared memory holds the matrix as two float arrays
+// The same computation in double-float, for spin blocks of more than kSlaterRegMaxBlock electrons
+// (smaller ones: slater_reg.cu, the matrix in registers).  Shared memory holds the matrix as two float arrays
 // Ah, Al of [n][ns] with ns = n rounded up to even, plus 2 (zero padding columns stay zero
 // through the elimination), so that column pairs (j, j+1) are one 8-byte word of each.
 template <typename T, int NT>
-__global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) slater_df_kernel(const SlaterArgs a)
+__global__ void __launch_bounds__(NT) slater_df_kernel(const SlaterArgs a)
 {
     extern __shared__ float fsm[];
     __shared__ double red[NT / 32];
@@ -988,16 +962,14 @@ template <typename T>
 int launch_slater(const SlaterArgs& a, int nmax, cudaStream_t st)
 {
     if (a.arith == 1) {
+        if (nmax <= kSlaterRegMaxBlock)
+            return sizeof(T) == 8 ? launch_slater_reg_f64(a, nmax, st) : launch_slater_reg_f32(a, nmax, st);
         const int ns = ((nmax + 1) & ~1) + 2;
         const size_t smem = 2 * (size_t)nmax * ns * sizeof(float);
-        // blocks that fit twice in shared memory: two 256-thread CTAs per SM, as for the
-        // complex double-float kernel (static shared memory under 9 KB; 227 KB per SM)
-        const bool two = 2 * (smem + 9 * 1024) <= 227 * 1024;
-        auto k = two ? slater_df_kernel<T, 256> : slater_df_kernel<T, kSlaterDfThreads>;
-        const int nt = two ? 256 : kSlaterDfThreads;
+        auto k = slater_df_kernel<T, kSlaterDfThreads>;
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute(slater_df_kernel)");
-        k<<<(unsigned)a.n_walkers, nt, smem, st>>>(a);
+        k<<<(unsigned)a.n_walkers, kSlaterDfThreads, smem, st>>>(a);
         return cuda_error(cudaGetLastError(), "slater_df_kernel launch");
     }
     const size_t smem = (size_t)nmax * (nmax + 1) * sizeof(double);
