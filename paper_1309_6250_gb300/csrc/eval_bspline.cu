@@ -160,9 +160,9 @@ __device__ __forceinline__ void bspline_warp_task(const EvalArgs& p, long long w
 }
 
 // The same computation for float and bfloat16 tables with packed FP32 arithmetic
-// (fma.rn.f32x2: two orbitals per instruction) and the next stencil column's rows
+// (fma.rn.f32x2: two orbitals per instruction) and the rows of the next AHEAD stencil columns
 // loaded before the current column is contracted.
-template <typename T, bool LAPTAB>
+template <typename T, bool LAPTAB, int AHEAD>
 __device__ __forceinline__ void bspline_warp_task_x2(const EvalArgs& p, long long w0, int lane)
 {
     constexpr int E = Traits<T>::E;          // orbitals per lane (4 float, 8 bfloat16)
@@ -220,29 +220,23 @@ __device__ __forceinline__ void bspline_warp_task_x2(const EvalArgs& p, long lon
 #pragma unroll
     for (int j = 0; j < NP; ++j) V[j] = GX[j] = GY[j] = GZ[j] = LP[j] = 0ull;
 
-    uint4 cur[R], nxt[R];
-    {
-        const size_t col = (size_t)(xs[0] * p.ny + ys[0]) * colb;
+    uint4 ring[AHEAD + 1][R];   // column c in slot c mod (AHEAD + 1)
+    auto load_column = [&](int c) {
+        const size_t col = (size_t)(xs[c >> 2] * p.ny + ys[c & 3]) * colb;
 #pragma unroll
-        for (int n = 0; n < 4; ++n) cur[n] = ldg_table(p, t0 + col + n * rowb);
+        for (int n = 0; n < 4; ++n) ring[c % (AHEAD + 1)][n] = ldg_table(p, t0 + col + n * rowb);
         if (LAPTAB) {
 #pragma unroll
-            for (int n = 0; n < 4; ++n) cur[4 + n] = ldg_table(p, t1 + col + n * rowb);
+            for (int n = 0; n < 4; ++n) ring[c % (AHEAD + 1)][4 + n] = ldg_table(p, t1 + col + n * rowb);
         }
-    }
+    };
+#pragma unroll
+    for (int c = 0; c < AHEAD; ++c) load_column(c);
 #pragma unroll
     for (int c = 0; c < 16; ++c) {
         const int l = c >> 2, m = c & 3;
-        if (c < 15) {   // next column's rows in flight while this one is contracted
-            const int ln = (c + 1) >> 2, mn = (c + 1) & 3;
-            const size_t col = (size_t)(xs[ln] * p.ny + ys[mn]) * colb;
-#pragma unroll
-            for (int n = 0; n < 4; ++n) nxt[n] = ldg_table(p, t0 + col + n * rowb);
-            if (LAPTAB) {
-#pragma unroll
-                for (int n = 0; n < 4; ++n) nxt[4 + n] = ldg_table(p, t1 + col + n * rowb);
-            }
-        }
+        if (c + AHEAD < 16) load_column(c + AHEAD);
+        const uint4(&cur)[R] = ring[c % (AHEAD + 1)];
         f32x2 A0[NP], A1[NP], A2[NP], AL[NP];
 #pragma unroll
         for (int j = 0; j < NP; ++j) A0[j] = A1[j] = A2[j] = AL[j] = 0ull;
@@ -282,10 +276,6 @@ __device__ __forceinline__ void bspline_warp_task_x2(const EvalArgs& p, long lon
 #pragma unroll
             for (int j = 0; j < NP; ++j) LP[j] = ffma2(C0, A0[j], ffma2(C1, A1[j], ffma2(C2, A2[j], LP[j])));
         }
-        if (c < 15) {
-#pragma unroll
-            for (int k = 0; k < R; ++k) cur[k] = nxt[k];
-        }
     }
 
     const int o0 = chunk * E;
@@ -321,7 +311,7 @@ __device__ __forceinline__ void bspline_warp_task_x2(const EvalArgs& p, long lon
 // product and sum carried as a double-float pair on the FP32 pipe (see df_fma2), results
 // converted to double at the store.
 
-template <bool LAPTAB>
+template <bool LAPTAB, int UNROLL>
 __device__ __forceinline__ void bspline_warp_task_df(const EvalArgs& p, long long w0, int lane)
 {
     const int L = 1 << p.lanes_log2;
@@ -377,7 +367,7 @@ __device__ __forceinline__ void bspline_warp_task_df(const EvalArgs& p, long lon
                             : nullptr;
     // accumulators (h, l) for value, reduced gradient, Laplacian-table value
     f32x2 Vh = 0, Vl = 0, Xh = 0, Xl = 0, Yh = 0, Yl = 0, Zh = 0, Zl = 0, Lh = 0, Ll = 0;
-#pragma unroll 1
+#pragma unroll UNROLL
     for (int c = 0; c < 16; ++c) {
         const int l = c >> 2, m = c & 3;
         const size_t col = (size_t)(xs[l] * p.ny + ys[m]) * colb;
@@ -487,13 +477,14 @@ __device__ __forceinline__ void bspline_warp_task_df(const EvalArgs& p, long lon
     if (p.lap) store_run<double, E>(static_cast<double*>(p.lap) + ip * p.n_orb + o0, lp, o0, p.n_orb, vec);
 }
 
-// float and bfloat16 tables take the packed path, double tables the scalar one
-template <typename T, bool LAPTAB>
+// float and bfloat16 tables take the packed path, double tables the scalar one.  AHEAD: columns of
+// rows in flight (packed path; columns unrolled for double-float tables).
+template <typename T, bool LAPTAB, int AHEAD = 1>
 __device__ __forceinline__ void warp_task(const EvalArgs& p, long long w0, int lane)
 {
-    if constexpr (std::is_same<T, DF64Tag>::value) bspline_warp_task_df<LAPTAB>(p, w0, lane);
+    if constexpr (std::is_same<T, DF64Tag>::value) bspline_warp_task_df<LAPTAB, AHEAD>(p, w0, lane);
     else if constexpr (sizeof(T) == 8) bspline_warp_task<T, LAPTAB>(p, w0, lane);
-    else bspline_warp_task_x2<T, LAPTAB>(p, w0, lane);
+    else bspline_warp_task_x2<T, LAPTAB, AHEAD>(p, w0, lane);
 }
 
 #ifndef QMCSPL_EVAL_THREADS
@@ -530,6 +521,17 @@ __global__ void __launch_bounds__(THREADS, 1) bspline_vgl_kernel(const EvalArgs 
     const long long wstride = (long long)gridDim.x * WPB;
     for (long long w0 = warp * gpw; w0 < total; w0 += wstride * gpw)
         warp_task<T, LAPTAB>(p, w0, lane);
+}
+
+// Launches of at most kSmallWarps warp tasks per SM: a block per warp task, so that they spread over
+// all SMs, and three columns of rows in flight (the registers of the missing warps are free), since
+// nothing but a warp's own loads hides their latency.
+constexpr int kSmallAhead = 3;
+template <typename T, bool LAPTAB>
+__global__ void __launch_bounds__(32) bspline_vgl_small_kernel(const EvalArgs p)
+{
+    const long long w0 = (long long)blockIdx.x << (5 - p.lanes_log2);
+    warp_task<T, LAPTAB, kSmallAhead>(p, w0, threadIdx.x);
 }
 
 // Several cells in one launch: warp task w belongs to the cell c with
@@ -579,12 +581,19 @@ int launch_shape(const EvalArgs& a, long long warps, cudaStream_t st)
     return cuda_error(cudaGetLastError(), "bspline_vgl_kernel launch");
 }
 
+template <typename T, bool LAPTAB>
+int launch_small(const EvalArgs& a, long long warps, cudaStream_t st)
+{
+    bspline_vgl_small_kernel<T, LAPTAB><<<(unsigned)warps, 32, 0, st>>>(a);
+    return cuda_error(cudaGetLastError(), "bspline_vgl_small_kernel launch");
+}
+
 // Block shapes a caller may choose (qmcspl_set_block, the batched launch plan): 512 threads for
 // every table type, 640 for float and bfloat16 tables (96 registers).
 template <typename T> constexpr bool kHas640 = std::is_same<T, float>::value || std::is_same<T, __nv_bfloat16>::value;
 
-// `threads` = 0: the automatic rule (the large shape from kLargeLaunchRounds rounds of warp tasks
-// on); 512 or 640: that shape.
+// `threads` = 0: the automatic rule (the small kernel up to kSmallWarps warp tasks per SM, the large
+// shape from kLargeLaunchRounds rounds of warp tasks on); 512 or 640: that shape.
 template <typename T, bool LAPTAB>
 int launch_typed(const EvalArgs& a, int threads, cudaStream_t st)
 {
@@ -594,6 +603,7 @@ int launch_typed(const EvalArgs& a, int threads, cudaStream_t st)
         if (threads == 640) return launch_shape<T, LAPTAB, 640>(a, warps, st);
     }
     if (threads == QMCSPL_EVAL_THREADS) return launch_shape<T, LAPTAB, QMCSPL_EVAL_THREADS>(a, warps, st);
+    if (small_launch(warps)) return launch_small<T, LAPTAB>(a, warps, st);
     constexpr int large = BspBlock<T, LAPTAB>::large;
     if constexpr (large != QMCSPL_EVAL_THREADS) {
         if (warps >= (long long)kLargeLaunchRounds * sm_count() * (large / 32))

@@ -89,8 +89,9 @@ __global__ void __launch_bounds__(kEvalThreads, DEG == 1 ? 1 : 2) general_vgl_ke
     const int sub = lane & (L - 1);
     const int gpw = 32 >> p.lanes_log2;
     const long long total = p.n_pos * p.tiles;
-    const long long warp = (long long)blockIdx.x * (kEvalThreads / 32) + (threadIdx.x >> 5);
-    const long long wstride = (long long)gridDim.x * (kEvalThreads / 32);
+    const int wpb = blockDim.x >> 5;   // 8, or 1 in small launches
+    const long long warp = (long long)blockIdx.x * wpb + (threadIdx.x >> 5);
+    const long long wstride = (long long)gridDim.x * wpb;
     const size_t rowb = (size_t)p.row_stride * sizeof(T);
     const size_t colb = (size_t)p.col_stride * sizeof(T);
     const A* mgv;
@@ -302,6 +303,10 @@ int launch_one(const EvalArgs& a, bool laptab, cudaStream_t st)
     void (*k)(EvalArgs) = laptab ? general_vgl_kernel<T, DEG, NONUNI, true> : general_vgl_kernel<T, DEG, NONUNI, false>;
     const int gpw = 32 >> a.lanes_log2;
     const long long warps = (a.n_pos * a.tiles + gpw - 1) / gpw;
+    if (small_launch(warps)) {
+        k<<<(unsigned)warps, 32, 0, st>>>(a);
+        return cuda_error(cudaGetLastError(), "general_vgl_kernel launch");
+    }
     long long blocks = (warps + kEvalThreads / 32 - 1) / (kEvalThreads / 32);
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kEvalThreads, 0);

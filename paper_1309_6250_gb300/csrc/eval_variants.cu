@@ -618,11 +618,16 @@ __global__ void __launch_bounds__(THREADS, 1) pp_vgl_kernel(const EvalArgs p)
     }
 }
 
+// `small`: the same kernel with a block per warp task, for small launches
 template <typename K>
-int launch_one_block_per_sm(K kernel, int threads, const EvalArgs& a, cudaStream_t st, const char* name)
+int launch_one_block_per_sm(K kernel, K small, int threads, const EvalArgs& a, cudaStream_t st, const char* name)
 {
     const int gpw = 32 >> a.lanes_log2;
     const long long warps = (a.n_pos * a.tiles + gpw - 1) / gpw;
+    if (small_launch(warps)) {
+        small<<<(unsigned)warps, 32, 0, st>>>(a);
+        return cuda_error(cudaGetLastError(), name);
+    }
     long long blocks = (warps + threads / 32 - 1) / (threads / 32);
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
@@ -638,15 +643,16 @@ int launch_one_block_per_sm(K kernel, int threads, const EvalArgs& a, cudaStream
 template <typename T, int BASIS>
 int launch_five(const EvalArgs& a, cudaStream_t st)
 {
-    return launch_one_block_per_sm(five_table_vgl_kernel<T, BASIS, QMCSPL_FIVE_THREADS>, QMCSPL_FIVE_THREADS, a, st,
+    return launch_one_block_per_sm(five_table_vgl_kernel<T, BASIS, QMCSPL_FIVE_THREADS>,
+                                   five_table_vgl_kernel<T, BASIS, 32>, QMCSPL_FIVE_THREADS, a, st,
                                    "five_table_vgl_kernel launch");
 }
 
 template <typename T>
 int launch_pp(const EvalArgs& a, cudaStream_t st)
 {
-    return launch_one_block_per_sm(pp_vgl_kernel<T, QMCSPL_FIVE_THREADS>, QMCSPL_FIVE_THREADS, a, st,
-                                   "pp_vgl_kernel launch");
+    return launch_one_block_per_sm(pp_vgl_kernel<T, QMCSPL_FIVE_THREADS>, pp_vgl_kernel<T, 32>, QMCSPL_FIVE_THREADS, a,
+                                   st, "pp_vgl_kernel launch");
 }
 
 EvalArgs make_args(const Handle* h, const double* pos, const Prepared& pr, long long n_pos, void* val,

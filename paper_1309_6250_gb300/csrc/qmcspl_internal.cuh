@@ -248,6 +248,10 @@ void fill_eval_args(const Handle* h, EvalArgs* a);
 
 // number of SMs of the current device (cached)
 int sm_count();
+// Evaluation launches of at most this many warp tasks per SM run one task per block: blocks of 8 or
+// 16 warps would leave them on a few SMs.
+constexpr int kSmallWarps = 8;
+inline bool small_launch(long long warps) { return warps <= (long long)kSmallWarps * sm_count(); }
 long long l2_cache_bytes();   // L2 size of the current device
 
 }  // namespace qmcspl
