@@ -162,8 +162,9 @@ __device__ __forceinline__ void bspline_warp_task(const EvalArgs& p, long long w
 // The same computation for float and bfloat16 tables with packed FP32 arithmetic
 // (fma.rn.f32x2: two orbitals per instruction) and the rows of the next AHEAD stencil columns
 // loaded before the current column is contracted.
-template <typename T, bool LAPTAB, int AHEAD>
-__device__ __forceinline__ void bspline_warp_task_x2(const EvalArgs& p, long long w0, int lane)
+// stage: with RAGGED, the warp's shared memory for the stores of unaligned rows (see RaggedStore).
+template <typename T, bool LAPTAB, int AHEAD, bool RAGGED>
+__device__ __forceinline__ void bspline_warp_task_x2(const EvalArgs& p, long long w0, int lane, float* stage)
 {
     constexpr int E = Traits<T>::E;          // orbitals per lane (4 float, 8 bfloat16)
     constexpr int NP = Pairs<T>::N;          // packed pairs per lane
@@ -186,8 +187,8 @@ __device__ __forceinline__ void bspline_warp_task_x2(const EvalArgs& p, long lon
     // (the bfloat16 kernel runs fastest with the rolled form of the reduction, the float one with
     // the written-out form; both give the same bits)
     coords_float<std::is_same<T, __nv_bfloat16>::value>(p, ip, L, sub, gbase, ix, iy, iz, tx, ty, tz, ok);
-    if (!active) return;
-    if (!ok && sub == 0 && tile == 0) atomicOr(p.err, 1);
+    if (!RAGGED && !active) return;   // (all lanes take part in the staged stores)
+    if (active && !ok && sub == 0 && tile == 0) atomicOr(p.err, 1);
 
     float bx[4], dbx[4], d2bx[4], by[4], dby[4], d2by[4], bz[4], dbz[4], d2bz[4];
     bspline_weights<float>(tx, bx, dbx, LAPTAB ? nullptr : d2bx);
@@ -279,7 +280,7 @@ __device__ __forceinline__ void bspline_warp_task_x2(const EvalArgs& p, long lon
     }
 
     const int o0 = chunk * E;
-    if (o0 >= p.n_orb) return;
+    if (!RAGGED && o0 >= p.n_orb) return;
     const bool vec = p.vec_out != 0;
     float v[E], gx[E], gy[E], gz[E], lp[E];
 #pragma unroll
@@ -298,6 +299,15 @@ __device__ __forceinline__ void bspline_warp_task_x2(const EvalArgs& p, long lon
         for (int e = 0; e < E; ++e) cg[a][e] = fmaf(m0, gx[e], fmaf(m1, gy[e], m2 * gz[e]));
     }
     if (p.phase) bloch_apply<float, E>(p, ip, v, cg, lp, true, !LAPTAB);
+    if constexpr (RAGGED) {
+        RaggedStore<E> out(stage, ip, o0, active, p.n_orb);
+        if (p.val) out.put(static_cast<float*>(p.val), v, 1, 0);
+        if (p.grad)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) out.put(static_cast<float*>(p.grad), cg[a], 3, a);
+        if (p.lap) out.put(static_cast<float*>(p.lap), lp, 1, 0);
+        return;
+    }
     if (p.val) store_run<float, E>(static_cast<float*>(p.val) + ip * p.n_orb + o0, v, o0, p.n_orb, vec);
     if (p.grad) {
         float* g = static_cast<float*>(p.grad) + ip * 3 * p.n_orb + o0;
@@ -479,12 +489,12 @@ __device__ __forceinline__ void bspline_warp_task_df(const EvalArgs& p, long lon
 
 // float and bfloat16 tables take the packed path, double tables the scalar one.  AHEAD: columns of
 // rows in flight (packed path; columns unrolled for double-float tables).
-template <typename T, bool LAPTAB, int AHEAD = 1>
-__device__ __forceinline__ void warp_task(const EvalArgs& p, long long w0, int lane)
+template <typename T, bool LAPTAB, int AHEAD = 1, bool RAGGED = false>
+__device__ __forceinline__ void warp_task(const EvalArgs& p, long long w0, int lane, float* stage = nullptr)
 {
     if constexpr (std::is_same<T, DF64Tag>::value) bspline_warp_task_df<LAPTAB, AHEAD>(p, w0, lane);
     else if constexpr (sizeof(T) == 8) bspline_warp_task<T, LAPTAB>(p, w0, lane);
-    else bspline_warp_task_x2<T, LAPTAB, AHEAD>(p, w0, lane);
+    else bspline_warp_task_x2<T, LAPTAB, AHEAD, RAGGED>(p, w0, lane, stage);
 }
 
 #ifndef QMCSPL_EVAL_THREADS
@@ -510,28 +520,30 @@ template <> struct BspBlock<float, true> {
 };
 constexpr int kLargeLaunchRounds = 4;   // warp-task rounds from which the large shape is used
 
-template <typename T, bool LAPTAB, int THREADS>
+template <typename T, bool LAPTAB, int THREADS, bool RAGGED>
 __global__ void __launch_bounds__(THREADS, 1) bspline_vgl_kernel(const EvalArgs p)
 {
     constexpr int WPB = THREADS / 32;
+    __shared__ __align__(16) float stage[RAGGED ? WPB : 1][kStageFloats<T, RAGGED>];
     const int lane = threadIdx.x & 31;
     const int gpw = 32 >> p.lanes_log2;
     const long long total = p.n_pos * p.tiles;
     const long long warp = (long long)blockIdx.x * WPB + (threadIdx.x >> 5);
     const long long wstride = (long long)gridDim.x * WPB;
     for (long long w0 = warp * gpw; w0 < total; w0 += wstride * gpw)
-        warp_task<T, LAPTAB>(p, w0, lane);
+        warp_task<T, LAPTAB, 1, RAGGED>(p, w0, lane, stage[RAGGED ? threadIdx.x >> 5 : 0]);
 }
 
 // Launches of at most kSmallWarps warp tasks per SM: a block per warp task, so that they spread over
 // all SMs, and three columns of rows in flight (the registers of the missing warps are free), since
 // nothing but a warp's own loads hides their latency.
 constexpr int kSmallAhead = 3;
-template <typename T, bool LAPTAB>
-__global__ void __launch_bounds__(32) bspline_vgl_small_kernel(const EvalArgs p)
+template <typename T, bool LAPTAB, bool RAGGED>
+__global__ void __launch_bounds__(32, kSmallWarps) bspline_vgl_small_kernel(const EvalArgs p)
 {
+    __shared__ __align__(16) float stage[kStageFloats<T, RAGGED>];
     const long long w0 = (long long)blockIdx.x << (5 - p.lanes_log2);
-    warp_task<T, LAPTAB, kSmallAhead>(p, w0, threadIdx.x);
+    warp_task<T, LAPTAB, kSmallAhead, RAGGED>(p, w0, threadIdx.x, stage);
 }
 
 // Several cells in one launch: warp task w belongs to the cell c with
@@ -576,15 +588,22 @@ long long grid_for(K kernel, int threads, long long warps)
 template <typename T, bool LAPTAB, int THREADS>
 int launch_shape(const EvalArgs& a, long long warps, cudaStream_t st)
 {
-    const long long blocks = grid_for(bspline_vgl_kernel<T, LAPTAB, THREADS>, THREADS, warps);
-    bspline_vgl_kernel<T, LAPTAB, THREADS><<<(unsigned)blocks, THREADS, 0, st>>>(a);
+    auto k = bspline_vgl_kernel<T, LAPTAB, THREADS, false>;
+    if constexpr (kStaged<T>) {
+        if (!a.vec_out) k = bspline_vgl_kernel<T, LAPTAB, THREADS, true>;
+    }
+    k<<<(unsigned)grid_for(k, THREADS, warps), THREADS, 0, st>>>(a);
     return cuda_error(cudaGetLastError(), "bspline_vgl_kernel launch");
 }
 
 template <typename T, bool LAPTAB>
 int launch_small(const EvalArgs& a, long long warps, cudaStream_t st)
 {
-    bspline_vgl_small_kernel<T, LAPTAB><<<(unsigned)warps, 32, 0, st>>>(a);
+    auto k = bspline_vgl_small_kernel<T, LAPTAB, false>;
+    if constexpr (kStaged<T>) {
+        if (!a.vec_out) k = bspline_vgl_small_kernel<T, LAPTAB, true>;
+    }
+    k<<<(unsigned)warps, 32, 0, st>>>(a);
     return cuda_error(cudaGetLastError(), "bspline_vgl_small_kernel launch");
 }
 

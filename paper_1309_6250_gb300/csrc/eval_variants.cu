@@ -136,8 +136,9 @@ __device__ __forceinline__ void five_table_task(const EvalArgs& p, long long w0,
 // position (16 columns x 5 tables, four z rows each) walked through a ring of three, so two
 // units' rows are in flight while one is contracted.  Same products and sums, in the same
 // order, as the scalar path.
-template <typename T, int BASIS>
-__device__ __forceinline__ void five_table_task_x2(const EvalArgs& p, long long w0, int lane)
+// RAGGED, stage: as the B-spline task's.
+template <typename T, int BASIS, bool RAGGED>
+__device__ __forceinline__ void five_table_task_x2(const EvalArgs& p, long long w0, int lane, float* stage)
 {
     constexpr int E = Traits<T>::E;
     constexpr int NP = Pairs<T>::N;
@@ -159,8 +160,8 @@ __device__ __forceinline__ void five_table_task_x2(const EvalArgs& p, long long 
     float tx, ty, tz;
     bool ok;
     coords_float(p, ip, L, sub, gbase, ix, iy, iz, tx, ty, tz, ok);
-    if (!active) return;
-    if (!ok && sub == 0 && tile == 0) atomicOr(p.err, 1);
+    if (!RAGGED && !active) return;   // (all lanes take part in the staged stores)
+    if (active && !ok && sub == 0 && tile == 0) atomicOr(p.err, 1);
     float lx[4], ly[4], lz[4];
     value_weights<BASIS, float>(tx, lx);
     value_weights<BASIS, float>(ty, ly);
@@ -210,7 +211,7 @@ __device__ __forceinline__ void five_table_task_x2(const EvalArgs& p, long long 
         for (int j = 0; j < NP; ++j) ACC[k][j] = ffma2(W, a[j], ACC[k][j]);
     }
     const int o0 = chunk * E;
-    if (o0 >= p.n_orb) return;
+    if (!RAGGED && o0 >= p.n_orb) return;
     const bool vec = p.vec_out != 0;
     float acc[5][E];
 #pragma unroll
@@ -218,6 +219,15 @@ __device__ __forceinline__ void five_table_task_x2(const EvalArgs& p, long long 
 #pragma unroll
         for (int j = 0; j < NP; ++j) unpack2(ACC[k][j], acc[k][2 * j], acc[k][2 * j + 1]);
     if (p.phase) bloch_apply<float, E>(p, ip, acc[0], acc + 1, acc[4], false, false);
+    if constexpr (RAGGED) {
+        RaggedStore<E> out(stage, ip, o0, active, p.n_orb);
+        if (p.val) out.put(static_cast<float*>(p.val), acc[0], 1, 0);
+        if (p.grad)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) out.put(static_cast<float*>(p.grad), acc[1 + a], 3, a);
+        if (p.lap) out.put(static_cast<float*>(p.lap), acc[4], 1, 0);
+        return;
+    }
     if (p.val) store_run<float, E>(static_cast<float*>(p.val) + ip * p.n_orb + o0, acc[0], o0, p.n_orb, vec);
     if (p.grad)
 #pragma unroll
@@ -331,10 +341,11 @@ __device__ __forceinline__ void five_table_task_df(const EvalArgs& p, long long 
 #endif
 // Five-table and pp kernels: one block of QMCSPL_FIVE_THREADS per SM, as the B-spline kernel: the warps of an SM evaluate consecutive
 // (cell-ordered, neighbouring) positions, whose stencil rows then hit in that SM's L1.
-template <typename T, int BASIS, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1) five_table_vgl_kernel(const EvalArgs p)
+template <typename T, int BASIS, int THREADS, bool RAGGED>
+__global__ void __launch_bounds__(THREADS, THREADS == 32 ? kSmallWarps : 1) five_table_vgl_kernel(const EvalArgs p)
 {
     constexpr int WPB = THREADS / 32;
+    __shared__ __align__(16) float stage[RAGGED ? WPB : 1][kStageFloats<T, RAGGED>];
     const int lane = threadIdx.x & 31;
     const int gpw = 32 >> p.lanes_log2;
     const long long total = p.n_pos * p.tiles;
@@ -343,7 +354,7 @@ __global__ void __launch_bounds__(THREADS, 1) five_table_vgl_kernel(const EvalAr
     for (long long w0 = warp * gpw; w0 < total; w0 += wstride * gpw) {
         if constexpr (std::is_same<T, DF64Tag>::value) five_table_task_df<BASIS>(p, w0, lane);
         else if constexpr (sizeof(T) == 8) five_table_task<T, BASIS>(p, w0, lane);
-        else five_table_task_x2<T, BASIS>(p, w0, lane);
+        else five_table_task_x2<T, BASIS, RAGGED>(p, w0, lane, stage[RAGGED ? threadIdx.x >> 5 : 0]);
     }
 }
 
@@ -476,8 +487,9 @@ __device__ __forceinline__ void pp_task(const EvalArgs& p, long long w0, int lan
 // float and bfloat16 tables: packed FP32 pairs, the 16 load units of a position (2 x 2
 // corner columns x 4 (kappa, mu) labels, four rows each: 2 z corners x 2 nu labels) through a
 // ring of three.  Same products and sums, in the same order, as the scalar path.
-template <typename T>
-__device__ __forceinline__ void pp_task_x2(const EvalArgs& p, long long w0, int lane)
+// RAGGED, stage: as the B-spline task's.
+template <typename T, bool RAGGED>
+__device__ __forceinline__ void pp_task_x2(const EvalArgs& p, long long w0, int lane, float* stage)
 {
     constexpr int E = Traits<T>::E;
     constexpr int NP = Pairs<T>::N;
@@ -500,8 +512,8 @@ __device__ __forceinline__ void pp_task_x2(const EvalArgs& p, long long w0, int 
     float tx, ty, tz;
     bool ok;
     coords_float(p, ip, L, sub, gbase, ix, iy, iz, tx, ty, tz, ok);
-    if (!active) return;
-    if (!ok && sub == 0 && tile == 0) atomicOr(p.err, 1);
+    if (!RAGGED && !active) return;   // (all lanes take part in the staged stores)
+    if (active && !ok && sub == 0 && tile == 0) atomicOr(p.err, 1);
     float wx[2][2], dwx[2][2], d2wx[2][2], wy[2][2], dwy[2][2], d2wy[2][2], wz[2][2], dwz[2][2], d2wz[2][2];
     pp_weights<float>(tx, wx, dwx, d2wx);
     pp_weights<float>(ty, wy, dwy, d2wy);
@@ -575,7 +587,7 @@ __device__ __forceinline__ void pp_task_x2(const EvalArgs& p, long long w0, int 
         }
     }
     const int o0 = chunk * E;
-    if (o0 >= p.n_orb) return;
+    if (!RAGGED && o0 >= p.n_orb) return;
     const bool vec = p.vec_out != 0;
     float v[E], gx[E], gy[E], gz[E], lp[E];
 #pragma unroll
@@ -594,6 +606,15 @@ __device__ __forceinline__ void pp_task_x2(const EvalArgs& p, long long w0, int 
         for (int e = 0; e < E; ++e) cg[a][e] = fmaf(m0, gx[e], fmaf(m1, gy[e], m2 * gz[e]));
     }
     if (p.phase) bloch_apply<float, E>(p, ip, v, cg, lp, true, true);
+    if constexpr (RAGGED) {
+        RaggedStore<E> out(stage, ip, o0, active, p.n_orb);
+        if (p.val) out.put(static_cast<float*>(p.val), v, 1, 0);
+        if (p.grad)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) out.put(static_cast<float*>(p.grad), cg[a], 3, a);
+        if (p.lap) out.put(static_cast<float*>(p.lap), lp, 1, 0);
+        return;
+    }
     if (p.val) store_run<float, E>(static_cast<float*>(p.val) + ip * p.n_orb + o0, v, o0, p.n_orb, vec);
     if (p.grad) {
         float* g = static_cast<float*>(p.grad) + ip * 3 * p.n_orb + o0;
@@ -603,10 +624,11 @@ __device__ __forceinline__ void pp_task_x2(const EvalArgs& p, long long w0, int 
     if (p.lap) store_run<float, E>(static_cast<float*>(p.lap) + ip * p.n_orb + o0, lp, o0, p.n_orb, vec);
 }
 
-template <typename T, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1) pp_vgl_kernel(const EvalArgs p)
+template <typename T, int THREADS, bool RAGGED>
+__global__ void __launch_bounds__(THREADS, THREADS == 32 ? kSmallWarps : 1) pp_vgl_kernel(const EvalArgs p)
 {
     constexpr int WPB = THREADS / 32;
+    __shared__ __align__(16) float stage[RAGGED ? WPB : 1][kStageFloats<T, RAGGED>];
     const int lane = threadIdx.x & 31;
     const int gpw = 32 >> p.lanes_log2;
     const long long total = p.n_pos * p.tiles;
@@ -614,7 +636,7 @@ __global__ void __launch_bounds__(THREADS, 1) pp_vgl_kernel(const EvalArgs p)
     const long long wstride = (long long)gridDim.x * WPB;
     for (long long w0 = warp * gpw; w0 < total; w0 += wstride * gpw) {
         if constexpr (sizeof(T) == 8) pp_task<T>(p, w0, lane);
-        else pp_task_x2<T>(p, w0, lane);
+        else pp_task_x2<T, RAGGED>(p, w0, lane, stage[RAGGED ? threadIdx.x >> 5 : 0]);
     }
 }
 
@@ -640,19 +662,37 @@ int launch_one_block_per_sm(K kernel, K small, int threads, const EvalArgs& a, c
     return cuda_error(cudaGetLastError(), name);
 }
 
+template <typename T, int BASIS, bool RAGGED>
+int launch_five_rows(const EvalArgs& a, cudaStream_t st)
+{
+    return launch_one_block_per_sm(five_table_vgl_kernel<T, BASIS, QMCSPL_FIVE_THREADS, RAGGED>,
+                                   five_table_vgl_kernel<T, BASIS, 32, RAGGED>, QMCSPL_FIVE_THREADS, a, st,
+                                   "five_table_vgl_kernel launch");
+}
+
 template <typename T, int BASIS>
 int launch_five(const EvalArgs& a, cudaStream_t st)
 {
-    return launch_one_block_per_sm(five_table_vgl_kernel<T, BASIS, QMCSPL_FIVE_THREADS>,
-                                   five_table_vgl_kernel<T, BASIS, 32>, QMCSPL_FIVE_THREADS, a, st,
-                                   "five_table_vgl_kernel launch");
+    if constexpr (kStaged<T>) {
+        if (!a.vec_out) return launch_five_rows<T, BASIS, true>(a, st);
+    }
+    return launch_five_rows<T, BASIS, false>(a, st);
+}
+
+template <typename T, bool RAGGED>
+int launch_pp_rows(const EvalArgs& a, cudaStream_t st)
+{
+    return launch_one_block_per_sm(pp_vgl_kernel<T, QMCSPL_FIVE_THREADS, RAGGED>, pp_vgl_kernel<T, 32, RAGGED>,
+                                   QMCSPL_FIVE_THREADS, a, st, "pp_vgl_kernel launch");
 }
 
 template <typename T>
 int launch_pp(const EvalArgs& a, cudaStream_t st)
 {
-    return launch_one_block_per_sm(pp_vgl_kernel<T, QMCSPL_FIVE_THREADS>, pp_vgl_kernel<T, 32>, QMCSPL_FIVE_THREADS, a,
-                                   st, "pp_vgl_kernel launch");
+    if constexpr (kStaged<T>) {
+        if (!a.vec_out) return launch_pp_rows<T, true>(a, st);
+    }
+    return launch_pp_rows<T, false>(a, st);
 }
 
 EvalArgs make_args(const Handle* h, const double* pos, const Prepared& pr, long long n_pos, void* val,
