@@ -32,6 +32,23 @@ def _ptr(t: Optional[torch.Tensor]) -> ctypes.c_void_p:
     return ctypes.c_void_p(0 if t is None else t.data_ptr())
 
 
+def _raw_stream(stream: Optional[torch.cuda.Stream], device: torch.device) -> int:
+    """cudaStream_t of `stream`, or of the current stream of `device` (whichever device is current)."""
+    if stream is not None:
+        return stream.cuda_stream
+    index = device.index
+    return _current_raw_stream(torch.cuda.current_device() if index is None else index)
+
+
+# the handle itself where torch offers it (0.1 us; a Stream object costs 3 us, on calls of 8 us)
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream",
+                              lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
+def _addr(t: Optional[torch.Tensor]):
+    return None if t is None else t.data_ptr()
+
+
 _COMPLEX = {torch.float32: torch.complex64, torch.float64: torch.complex128}
 
 
@@ -90,6 +107,11 @@ class OrbitalSplines:
         self.n_fun = self.n_orb * (2 if self.bloch else 1)     # stored real functions per row
         self.out_dtype = torch.float64 if storage in ("f64", "df64") else torch.float32
         self.result_dtype = _COMPLEX[self.out_dtype] if self.bloch else self.out_dtype
+        # what a handle keeps for life: coefficient tables of a five-table or pp handle (else 0), and
+        # whether a single-spline handle has a Laplacian table
+        inf = self.info()
+        self.n_multi = 5 if inf["n_tables"] == 5 else (8 if inf["entries_per_point"] == 8 else 0)
+        self.lap_table = bool(inf["separate_lap"]) and not self.n_multi
 
     @classmethod
     def load(cls, path: str, device: Optional[torch.device] = None,
@@ -207,6 +229,8 @@ class OrbitalSplines:
     def _check_pos(self, pos: torch.Tensor) -> torch.Tensor:
         if pos.device != self.device or pos.dtype != torch.float64:
             raise ValueError("positions must be a float64 tensor on %s" % self.device)
+        if pos.dim() == 2 and pos.shape[1] == 3 and pos.is_contiguous():
+            return pos
         return pos.reshape(-1, 3).contiguous()
 
     def eval_vgl(self, pos: torch.Tensor, out=None, stream=None,
@@ -215,10 +239,12 @@ class OrbitalSplines:
         pos = self._check_pos(pos)
         n = pos.shape[0]
         val, grad, lap = out if out is not None else self.alloc_outputs(n)
-        with torch.cuda.device(self.device):
-            _lib.check(self.lib.qmcspl_eval_vgl(
-                self.handle, _ptr(pos), n, _ptr(val if want[0] else None),
-                _ptr(grad if want[1] else None), _ptr(lap if want[2] else None), _stream_handle(stream)))
+        # (the library switches to the handle's device itself)
+        rc = self.lib.qmcspl_eval_vgl(self.handle, pos.data_ptr(), n, _addr(val) if want[0] else None,
+                                      _addr(grad) if want[1] else None, _addr(lap) if want[2] else None,
+                                      _raw_stream(stream, self.device))
+        if rc:
+            _lib.check(rc)
         return val, grad, lap
 
     def eval_vgl_host(self, pos: torch.Tensor, out=None, stream=None, out_dtype=None):
@@ -256,10 +282,11 @@ class OrbitalSplines:
         # complex upstream gradients (Bloch handles) may carry a lazy conjugation bit
         c = lambda t: None if t is None else (t.resolve_conj() if t.is_complex() else t).contiguous()
         gv, gg, gl = c(gv), c(gg), c(gl)
-        with torch.cuda.device(self.device):
-            _lib.check(self.lib.qmcspl_eval_vgl_backward(
-                self.handle, _ptr(pos), n, _ptr(gv), _ptr(gg), _ptr(gl), _ptr(dcoef), _ptr(dcoef_lap),
-                _ptr(dpos), _stream_handle(stream)))
+        rc = self.lib.qmcspl_eval_vgl_backward(self.handle, pos.data_ptr(), n, _addr(gv), _addr(gg), _addr(gl),
+                                               _addr(dcoef), _addr(dcoef_lap), _addr(dpos),
+                                               _raw_stream(stream, self.device))
+        if rc:
+            _lib.check(rc)
         return dpos
 
     def coef_shape(self) -> Tuple[int, int, int, int]:

@@ -73,10 +73,8 @@ class SplineOrbitalFunction(torch.autograd.Function):
         (pos,) = ctx.saved_tensors
         need_pos = ctx.needs_input_grad[0]
         need_coef = ctx.needs_input_grad[1] or ctx.needs_input_grad[2]
-        inf = spl.info()
         # Lagrange and B-splines with separate gradient tables: five tables; pp: eight entries
-        n_multi = 5 if inf["n_tables"] == 5 else (8 if inf["entries_per_point"] == 8 else 0)
-        sep = bool(inf["separate_lap"]) and not n_multi
+        n_multi, sep = spl.n_multi, spl.lap_table
         dcoef = dcoef_lap = None
         if need_coef:
             shape = ((n_multi,) if n_multi else ()) + spl.coef_shape()
