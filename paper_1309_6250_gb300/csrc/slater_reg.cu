@@ -78,20 +78,19 @@ __device__ __forceinline__ void eliminate2(f32x2& H, f32x2& L, f32x2 fh, f32x2 f
     quick_norm2(H, L);
 }
 
-// (H, L) += x y for double-float x = xh + xl and y = yh + yl (the low products with the cross terms
-// xl yh and, where WIDE, xh yl).  P = fl(xh yh) enters H through a two-sum, whose error is
-// (H - A) + (P + B) with B = H - S, A = S + B; the product's own rounding error joins the second
-// term in one multiply-add, xh yh + B (ten operations; the product and its error apart took twelve).
+// (H, L) += x y for double-float x = xh + xl and y = yh + yl (yl only where WIDE): df_fma2's steps
 template <bool WIDE>
-__device__ __forceinline__ void dot2(f32x2& H, f32x2& L, f32x2 xh, f32x2 xl, f32x2 yh, f32x2 yl)
+__device__ __forceinline__ void dot2(f32x2& H, f32x2& L, f32x2 xh, f32x2 nxh, f32x2 xl, f32x2 yh, f32x2 yl)
 {
-    const f32x2 S = add2(H, ffma2(xh, yh, 0ull));   // (a plain mul2 here is contracted with the sum)
-    const f32x2 B = sub2(H, S);
-    const f32x2 A = sub2(H, add2(S, B));
-    f32x2 E = ffma2(xh, yh, B);
+    const f32x2 nP = mul2(nxh, yh);
+    f32x2 E = ffma2(xh, yh, nP);
     if (WIDE) E = ffma2(xh, yl, E);
     E = ffma2(xl, yh, E);
-    L = add2(L, add2(A, E));
+    const f32x2 S = sub2(H, nP);
+    const f32x2 B = sub2(S, H);
+    const f32x2 T1 = sub2(H, sub2(S, B));
+    const f32x2 T2 = add2(nP, B);
+    L = add2(L, add2(sub2(T1, T2), E));
     H = S;
 }
 
@@ -412,15 +411,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32 * RegShape<G>::NW
                         const int jj = lane + 32 * t;
                         if (jj >= n) continue;
                         const float2 x = xt[(size_t)i * ld + jj];
-                        const f32x2 xh = pack2(x.x, x.x), xl = pack2(x.y, x.y);
+                        const f32x2 xh = pack2(x.x, x.x), nxh = pack2(-x.x, -x.x), xl = pack2(x.y, x.y);
                         float g[3][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, q[2] = {0.f, 0.f};
                         if (want_g)
 #pragma unroll
                             for (int c = 0; c < 3; ++c)
                                 split(__ldg(gp + ((base + i) * 3 + c) * O + jj), g[c][0], g[c][1]);
                         if (want_l) split(__ldg(lp + (base + i) * O + jj), q[0], q[1]);
-                        dot2<kWide>(Ah, Al, xh, xl, pack2(g[0][0], g[1][0]), pack2(g[0][1], g[1][1]));
-                        dot2<kWide>(Bh, Bl, xh, xl, pack2(g[2][0], q[0]), pack2(g[2][1], q[1]));
+                        dot2<kWide>(Ah, Al, xh, nxh, xl, pack2(g[0][0], g[1][0]), pack2(g[0][1], g[1][1]));
+                        dot2<kWide>(Bh, Bl, xh, nxh, xl, pack2(g[2][0], q[0]), pack2(g[2][1], q[1]));
                     }
                     warp_sum2(Ah, Al);
                     warp_sum2(Bh, Bl);
