@@ -318,7 +318,7 @@ __device__ __forceinline__ void bspline_warp_task_x2(const EvalArgs& p, long lon
 }
 
 // Double-float tables (DF64Tag chunks, see eval_common.cuh): the same stencil walk with every
-// product and sum carried as a double-float pair on the FP32 pipe (see df_fma2), results
+// product and sum carried as a double-float pair on the FP32 pipe (see df_mad2), results
 // converted to double at the store.
 
 template <bool LAPTAB, int UNROLL>
@@ -375,6 +375,7 @@ __device__ __forceinline__ void bspline_warp_task_df(const EvalArgs& p, long lon
     const char* t0 = static_cast<const char*>(p.tab[0]) + (size_t)chunk * 16 + (size_t)iz * rowb;
     const char* t1 = LAPTAB ? static_cast<const char*>(p.tab[1]) + (size_t)chunk * 16 + (size_t)iz * rowb
                             : nullptr;
+    const f32x2 zero = pack2(p.zero, p.zero);   // (see df_mad2)
     // accumulators (h, l) for value, reduced gradient, Laplacian-table value
     f32x2 Vh = 0, Vl = 0, Xh = 0, Xl = 0, Yh = 0, Yl = 0, Zh = 0, Zl = 0, Lh = 0, Ll = 0;
 #pragma unroll UNROLL
@@ -388,44 +389,46 @@ __device__ __forceinline__ void bspline_warp_task_df(const EvalArgs& p, long lon
 #pragma unroll
             for (int n = 0; n < 4; ++n) rawl[n] = ldg_table(p, t1 + col + n * rowb);
         }
-        f32x2 A0h = 0, A0l = 0, A1h = 0, A1l = 0, A2h = 0, A2l = 0, ALh = 0, ALl = 0;
+        f32x2 A0h, A0l, A1h, A1l, A2h, A2l, ALh, ALl;
 #pragma unroll
         for (int n = 0; n < 4; ++n) {
+            auto add = [&](f32x2& Ah, f32x2& Al, dfloat w, f32x2 Bh, f32x2 Bl) {
+                const f32x2 wh = pack2(w.h, w.h), wl = pack2(w.l, w.l);
+                if (n == 0) df_mul2(Ah, Al, wh, wl, Bh, Bl, zero);
+                else df_mad2(Ah, Al, wh, wl, Bh, Bl, zero);
+            };
             const f32x2 Bh = pack2u(raw[n].x, raw[n].y), Bl = pack2u(raw[n].z, raw[n].w);
-            const f32x2 wh = pack2(bz[n].h, bz[n].h), wl = pack2(bz[n].l, bz[n].l), nwh = pack2(-bz[n].h, -bz[n].h);
-            df_fma2(A0h, A0l, wh, wl, nwh, Bh, Bl);
-            const f32x2 dh = pack2(dbz[n].h, dbz[n].h), dl = pack2(dbz[n].l, dbz[n].l),
-                        ndh = pack2(-dbz[n].h, -dbz[n].h);
-            df_fma2(A1h, A1l, dh, dl, ndh, Bh, Bl);
-            if (!LAPTAB) {
-                const f32x2 eh = pack2(d2bz[n].h, d2bz[n].h), el = pack2(d2bz[n].l, d2bz[n].l),
-                            neh = pack2(-d2bz[n].h, -d2bz[n].h);
-                df_fma2(A2h, A2l, eh, el, neh, Bh, Bl);
-            }
-            if (LAPTAB) {
-                const f32x2 Ch = pack2u(rawl[n].x, rawl[n].y), Cl = pack2u(rawl[n].z, rawl[n].w);
-                df_fma2(ALh, ALl, wh, wl, nwh, Ch, Cl);
-            }
+            add(A0h, A0l, bz[n], Bh, Bl);
+            add(A1h, A1l, dbz[n], Bh, Bl);
+            if (!LAPTAB) add(A2h, A2l, d2bz[n], Bh, Bl);
+            if (LAPTAB) add(ALh, ALl, bz[n], pack2u(rawl[n].x, rawl[n].y), pack2u(rawl[n].z, rawl[n].w));
         }
         const dfloat w00 = df_mul(bx[l], by[m]), w10 = df_mul(dbx[l], by[m]), w01 = df_mul(bx[l], dby[m]);
-        const f32x2 h00 = pack2(w00.h, w00.h), l00 = pack2(w00.l, w00.l), n00 = pack2(-w00.h, -w00.h);
-        const f32x2 h10 = pack2(w10.h, w10.h), l10 = pack2(w10.l, w10.l), n10 = pack2(-w10.h, -w10.h);
-        const f32x2 h01 = pack2(w01.h, w01.h), l01 = pack2(w01.l, w01.l), n01 = pack2(-w01.h, -w01.h);
-        df_fma2(Vh, Vl, h00, l00, n00, A0h, A0l);
-        df_fma2(Xh, Xl, h10, l10, n10, A0h, A0l);
-        df_fma2(Yh, Yl, h01, l01, n01, A0h, A0l);
-        df_fma2(Zh, Zl, h00, l00, n00, A1h, A1l);
+        const f32x2 h00 = pack2(w00.h, w00.h), l00 = pack2(w00.l, w00.l);
+        const f32x2 h10 = pack2(w10.h, w10.h), l10 = pack2(w10.l, w10.l);
+        const f32x2 h01 = pack2(w01.h, w01.h), l01 = pack2(w01.l, w01.l);
+        df_mad2(Vh, Vl, h00, l00, A0h, A0l, zero);
+        df_mad2(Xh, Xl, h10, l10, A0h, A0l, zero);
+        df_mad2(Yh, Yl, h01, l01, A0h, A0l, zero);
+        df_mad2(Zh, Zl, h00, l00, A1h, A1l, zero);
         if (LAPTAB) {
-            df_fma2(Lh, Ll, h00, l00, n00, ALh, ALl);
+            df_mad2(Lh, Ll, h00, l00, ALh, ALl, zero);
         } else {
             // metric folded into per-column weights: lap += c0 A0 + c1 A1 + c2 A2
             const dfloat c0 = df_add(df_add(df_mul(ml[0], df_mul(d2bx[l], by[m])), df_mul(ml[1], df_mul(bx[l], d2by[m]))),
                                      df_mul(ml[3], df_mul(dbx[l], dby[m])));
             const dfloat c1 = df_add(df_mul(ml[4], w10), df_mul(ml[5], w01));
             const dfloat c2 = df_mul(ml[2], w00);
-            df_fma2(Lh, Ll, pack2(c0.h, c0.h), pack2(c0.l, c0.l), pack2(-c0.h, -c0.h), A0h, A0l);
-            df_fma2(Lh, Ll, pack2(c1.h, c1.h), pack2(c1.l, c1.l), pack2(-c1.h, -c1.h), A1h, A1l);
-            df_fma2(Lh, Ll, pack2(c2.h, c2.h), pack2(c2.l, c2.l), pack2(-c2.h, -c2.h), A2h, A2l);
+            df_mad2(Lh, Ll, pack2(c0.h, c0.h), pack2(c0.l, c0.l), A0h, A0l, zero);
+            df_mad2(Lh, Ll, pack2(c1.h, c1.h), pack2(c1.l, c1.l), A1h, A1l, zero);
+            df_mad2(Lh, Ll, pack2(c2.h, c2.h), pack2(c2.l, c2.l), A2h, A2l, zero);
+        }
+        if (m == 3) {
+            df_renorm2(Vh, Vl);
+            df_renorm2(Xh, Xl);
+            df_renorm2(Yh, Yl);
+            df_renorm2(Zh, Zl);
+            df_renorm2(Lh, Ll);
         }
     }
 
@@ -446,9 +449,9 @@ __device__ __forceinline__ void bspline_warp_task_df(const EvalArgs& p, long lon
             f32x2 Gh = 0, Gl = 0;
             const float m0h = p.mgh[3 * a], m1h = p.mgh[3 * a + 1], m2h = p.mgh[3 * a + 2];
             const float m0l = p.mgl[3 * a], m1l = p.mgl[3 * a + 1], m2l = p.mgl[3 * a + 2];
-            df_fma2(Gh, Gl, pack2(m0h, m0h), pack2(m0l, m0l), pack2(-m0h, -m0h), Xh, Xl);
-            df_fma2(Gh, Gl, pack2(m1h, m1h), pack2(m1l, m1l), pack2(-m1h, -m1h), Yh, Yl);
-            df_fma2(Gh, Gl, pack2(m2h, m2h), pack2(m2l, m2l), pack2(-m2h, -m2h), Zh, Zl);
+            df_mad2(Gh, Gl, pack2(m0h, m0h), pack2(m0l, m0l), Xh, Xl, zero);
+            df_mad2(Gh, Gl, pack2(m1h, m1h), pack2(m1l, m1l), Yh, Yl, zero);
+            df_mad2(Gh, Gl, pack2(m2h, m2h), pack2(m2l, m2l), Zh, Zl, zero);
             unpack2(Gh, a0, a1); unpack2(Gl, b0, b1);
             dg[a][0] = {a0, b0};
             dg[a][1] = {a1, b1};

@@ -238,7 +238,7 @@ __device__ __forceinline__ void five_table_task_x2(const EvalArgs& p, long long 
 }
 
 // Double-float tables (B-splines with separate gradient tables): every weight, product and sum
-// a double-float pair on the FP32 pipe (df_fma2, two orbitals per packed operation), as the
+// a double-float pair on the FP32 pipe (df_mad2, two orbitals per packed operation), as the
 // double-float B-spline kernel; the outputs are converted to double for the epilogue.
 template <int BASIS>
 __device__ __forceinline__ void five_table_task_df(const EvalArgs& p, long long w0, int lane)
@@ -287,6 +287,7 @@ __device__ __forceinline__ void five_table_task_df(const EvalArgs& p, long long 
     }
     const int chunk = tile * L + sub;
     const size_t off = (size_t)chunk * 16 + (size_t)iz * rowb;
+    const f32x2 zero = pack2(p.zero, p.zero);   // (see df_mad2)
     f32x2 Ah[5], Al[5];
 #pragma unroll
     for (int k = 0; k < 5; ++k) Ah[k] = Al[k] = 0ull;
@@ -295,21 +296,23 @@ __device__ __forceinline__ void five_table_task_df(const EvalArgs& p, long long 
         const int l = c >> 2, m = c & 3;
         const size_t col = (size_t)(xs[l] * p.ny + ys[m]) * colb + off;
         const dfloat wxy = df_mul(lw[0][l], lw[1][m]);
-        const f32x2 xh = pack2(wxy.h, wxy.h), xl = pack2(wxy.l, wxy.l), nxh = pack2(-wxy.h, -wxy.h);
+        const f32x2 xh = pack2(wxy.h, wxy.h), xl = pack2(wxy.l, wxy.l);
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
             const char* base = static_cast<const char*>(p.tab[k]) + col;
             uint4 raw[4];
 #pragma unroll
             for (int n = 0; n < 4; ++n) raw[n] = ldg_table(p, base + n * rowb);
-            f32x2 Sh = 0ull, Sl = 0ull;
+            f32x2 Sh, Sl;
 #pragma unroll
             for (int n = 0; n < 4; ++n) {
                 const f32x2 Bh = pack2u(raw[n].x, raw[n].y), Bl = pack2u(raw[n].z, raw[n].w);
                 const dfloat z = lw[2][n];
-                df_fma2(Sh, Sl, pack2(z.h, z.h), pack2(z.l, z.l), pack2(-z.h, -z.h), Bh, Bl);
+                if (n == 0) df_mul2(Sh, Sl, pack2(z.h, z.h), pack2(z.l, z.l), Bh, Bl, zero);
+                else df_mad2(Sh, Sl, pack2(z.h, z.h), pack2(z.l, z.l), Bh, Bl, zero);
             }
-            df_fma2(Ah[k], Al[k], xh, xl, nxh, Sh, Sl);
+            df_mad2(Ah[k], Al[k], xh, xl, Sh, Sl, zero);
+            if (m == 3) df_renorm2(Ah[k], Al[k]);
         }
     }
     constexpr int E = 2;

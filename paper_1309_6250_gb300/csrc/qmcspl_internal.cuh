@@ -67,6 +67,7 @@ struct EvalArgs {
     float mgf[9], mlf[6];     // the same rounded to float (float kernels)
     float mgh[9], mgl[9];     // double-float split of mg: mg = mgh + mgl
     float mlh[6], mll[6];     // double-float split of ml
+    float zero;               // 0, where the compiler must not know it (df_mad2)
     const double* pos;
     const void* rec;          // per-position coordinate records (null: compute from pos), see order.cu
     const int* perm;          // evaluation order: position perm[i] is the i-th evaluated (null: input order)
