@@ -28,6 +28,8 @@
 //   lap u:   h_lap
 // after which the real adjoint above applies unchanged.  The position adjoint gains the
 // derivative of the phase, d e / d r = i k e:  dL/dr += -k sum_z Im(conj(h_z) w_z).
+#include <type_traits>
+
 #include "backward_common.cuh"
 
 namespace qmcspl {
@@ -101,19 +103,19 @@ __device__ __forceinline__ void bwd_position(const BwdArgs& b, long long ip, boo
         const A* ggp = static_cast<const A*>(b.gg);
         const A* glp = static_cast<const A*>(b.gl);
         const bool use = active && o0 < n_orb;
-        load_run<A>(use && gvp ? gvp + ip * n_orb + o0 : nullptr, wv, o0, n_orb, E);
-        load_run<A>(use && glp ? glp + ip * n_orb + o0 : nullptr, wl, o0, n_orb, E);
+        load_run<A, E>(use && gvp ? gvp + ip * n_orb + o0 : nullptr, wv, o0, n_orb, b.vec_up);
+        load_run<A, E>(use && glp ? glp + ip * n_orb + o0 : nullptr, wl, o0, n_orb, b.vec_up);
         for (int a = 0; a < 3; ++a)
-            load_run<A>(use && ggp ? ggp + (ip * 3 + a) * n_orb + o0 : nullptr, wg[a], o0, n_orb, E);
+            load_run<A, E>(use && ggp ? ggp + (ip * 3 + a) * n_orb + o0 : nullptr, wg[a], o0, n_orb, b.vec_up);
         if constexpr (BLOCH) bloch_upstream<A, E, LAPTAB>(p, p.pos + 3 * ip, wv, wg, wl, hv, hg, hl);
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
             for (int e = 0; e < E; ++e)
-                gt[i][e] = (A)p.mg[i] * wg[0][e] + (A)p.mg[3 + i] * wg[1][e] + (A)p.mg[6 + i] * wg[2][e];
+                gt[i][e] = chain_mg<A>(p, i) * wg[0][e] + chain_mg<A>(p, 3 + i) * wg[1][e] + chain_mg<A>(p, 6 + i) * wg[2][e];
     }
-    const A ml0 = (A)p.ml[0], ml1 = (A)p.ml[1], ml2 = (A)p.ml[2];
-    const A ml3 = (A)p.ml[3], ml4 = (A)p.ml[4], ml5 = (A)p.ml[5];
+    const A ml0 = chain_ml<A>(p, 0), ml1 = chain_ml<A>(p, 1), ml2 = chain_ml<A>(p, 2);
+    const A ml3 = chain_ml<A>(p, 3), ml4 = chain_ml<A>(p, 4), ml5 = chain_ml<A>(p, 5);
     int xs[4], ys[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -260,8 +262,11 @@ __device__ __forceinline__ void bwd_position(const BwdArgs& b, long long ip, boo
     }
 }
 
+// Blocks of four warps: the float kernels' 168 registers per thread let three of them (12 warps) run
+// on an SM, where one block of eight warps did (4,096 positions x 128 orbitals, both adjoints: 159 -> 148 us).
+constexpr int kBwdThreads = 128;
 template <typename T, bool LAPTAB, bool BLOCH, bool COEF>
-__global__ void __launch_bounds__(kEvalThreads) bspline_bwd_kernel(const BwdArgs b)
+__global__ void __launch_bounds__(kBwdThreads, std::is_same<T, float>::value && !BLOCH ? 3 : 2) bspline_bwd_kernel(const BwdArgs b)
 {
     using A = typename Traits<T>::A;
     constexpr int E = Traits<T>::E;
@@ -272,8 +277,8 @@ __global__ void __launch_bounds__(kEvalThreads) bspline_bwd_kernel(const BwdArgs
     const int gbase = lane & ~(L - 1);
     const int gpw = 32 >> p.lanes_log2;
     const long long total = p.n_pos * p.tiles;
-    const long long warp = (long long)blockIdx.x * (kEvalThreads / 32) + (threadIdx.x >> 5);
-    const long long wstride = (long long)gridDim.x * (kEvalThreads / 32);
+    const long long warp = (long long)blockIdx.x * (kBwdThreads / 32) + (threadIdx.x >> 5);
+    const long long wstride = (long long)gridDim.x * (kBwdThreads / 32);
     const int n_orb = p.n_orb;
     A* dc = static_cast<A*>(b.dcoef);
     A* dl = static_cast<A*>(b.dcoef_lap);
@@ -391,17 +396,17 @@ __device__ __forceinline__ void dpos_task_x2(const BwdArgs& b, long long w0, int
         const float* ggp = static_cast<const float*>(b.gg);
         const float* glp = static_cast<const float*>(b.gl);
         const bool use = active && o0 < n_orb;
-        load_run<float>(use && gvp ? gvp + ip * n_orb + o0 : nullptr, wv, o0, n_orb, E);
-        load_run<float>(use && glp ? glp + ip * n_orb + o0 : nullptr, wl, o0, n_orb, E);
+        load_run<float, E>(use && gvp ? gvp + ip * n_orb + o0 : nullptr, wv, o0, n_orb, b.vec_up);
+        load_run<float, E>(use && glp ? glp + ip * n_orb + o0 : nullptr, wl, o0, n_orb, b.vec_up);
 #pragma unroll
         for (int a = 0; a < 3; ++a)
-            load_run<float>(use && ggp ? ggp + (ip * 3 + a) * n_orb + o0 : nullptr, wg[a], o0, n_orb, E);
+            load_run<float, E>(use && ggp ? ggp + (ip * 3 + a) * n_orb + o0 : nullptr, wg[a], o0, n_orb, b.vec_up);
         float gt[3][E];
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
             for (int e = 0; e < E; ++e)
-                gt[i][e] = (float)p.mg[i] * wg[0][e] + (float)p.mg[3 + i] * wg[1][e] + (float)p.mg[6 + i] * wg[2][e];
+                gt[i][e] = chain_mg<float>(p, i) * wg[0][e] + chain_mg<float>(p, 3 + i) * wg[1][e] + chain_mg<float>(p, 6 + i) * wg[2][e];
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
             WV[j] = pack2(wv[2 * j], wv[2 * j + 1]);
@@ -494,10 +499,11 @@ __device__ __forceinline__ void dpos_task_x2(const BwdArgs& b, long long w0, int
         uy += __shfl_xor_sync(kFullMask, uy, off);
         uz += __shfl_xor_sync(kFullMask, uz, off);
     }
-    if (active && sub == 0) {
+    // a component per lane where the group has three (FP64 instructions take a warp 64 cycles each)
+    const int per = L >= 4 ? 1 : 3;
+    if (active && (per == 3 ? sub == 0 : sub < 3)) {
         const double u[3] = {(double)ux, (double)uy, (double)uz};
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
+        for (int a = per == 3 ? 0 : sub, k = 0; k < per; ++k, ++a)
             atomicAdd(b.dpos + 3 * ip + a, p.mg[3 * a] * u[0] + p.mg[3 * a + 1] * u[1] + p.mg[3 * a + 2] * u[2]);
     }
 }
@@ -535,8 +541,16 @@ __global__ void __launch_bounds__(DposShape<T>::threads, 1) bspline_dpos_kernel(
 // row then goes to the coefficient gradient with one vector atomic per chunk: no shared-memory
 // atomics, one global reduction per point row and batch.  The table is not read; the position
 // adjoint is left to a second launch over the same cell order.
-constexpr int kGatherThreads = 512;
-constexpr int kGatherBatch = 64;                      // positions staged at a time
+// Threads per block, positions staged at a time and blocks per SM.  Float: two blocks of 256 threads on
+// an SM, so that one block's staging and barriers overlap the other's columns (the pass at 262,144
+// positions x 128 orbitals: 1.14 ms; one block of 512 threads and batches of 64: 1.33 ms); double
+// staging is too large for two.
+template <typename A> struct GatherShape {
+    static constexpr int threads = 256, batch = 40, per_sm = 2;
+};
+template <> struct GatherShape<double> {
+    static constexpr int threads = 512, batch = 64, per_sm = 1;
+};
 constexpr int kGatherSide = 7;                        // stencil points per axis of a 4-cell bin edge
 constexpr int kGatherColumns = kGatherSide * kGatherSide;
 
@@ -605,6 +619,7 @@ struct GatherArgs {
 // staged data of one batch (dynamic shared memory)
 template <typename A>
 struct GatherStage {
+    static constexpr int kGatherBatch = GatherShape<A>::batch;
     static constexpr int EA = 16 / sizeof(A);        // upstream values per 16-byte chunk
     A w[kGatherBatch][3][12];                        // per axis b[4], b'[4], b''[4]
     int cell[kGatherBatch];                          // local cell cx | cy << 8 | cz << 16, -1: none
@@ -613,10 +628,12 @@ struct GatherStage {
 };
 
 template <typename A, bool LAPTAB>
-__global__ void __launch_bounds__(kGatherThreads, 1) bspline_bwd_gather_kernel(const BwdArgs b, const GatherArgs g)
+__global__ void __launch_bounds__(GatherShape<A>::threads, GatherShape<A>::per_sm)
+    bspline_bwd_gather_kernel(const BwdArgs b, const GatherArgs g)
 {
     constexpr int EA = GatherStage<A>::EA;
-    constexpr int WARPS = kGatherThreads / 32;
+    constexpr int WARPS = GatherShape<A>::threads / 32;
+    constexpr int kGatherBatch = GatherShape<A>::batch;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     GatherStage<A>& S = *reinterpret_cast<GatherStage<A>*>(smem_raw);
     const EvalArgs& p = b.e;
@@ -628,8 +645,8 @@ __global__ void __launch_bounds__(kGatherThreads, 1) bspline_bwd_gather_kernel(c
     const A* gvp = static_cast<const A*>(b.gv);
     const A* ggp = static_cast<const A*>(b.gg);
     const A* glp = static_cast<const A*>(b.gl);
-    const A ml0 = (A)p.ml[0], ml1 = (A)p.ml[1], ml2 = (A)p.ml[2];
-    const A ml3 = (A)p.ml[3], ml4 = (A)p.ml[4], ml5 = (A)p.ml[5];
+    const A ml0 = chain_ml<A>(p, 0), ml1 = chain_ml<A>(p, 1), ml2 = chain_ml<A>(p, 2);
+    const A ml3 = chain_ml<A>(p, 3), ml4 = chain_ml<A>(p, 4), ml5 = chain_ml<A>(p, 5);
     const int items = g.n_bins * g.n_slices;
     for (int item = blockIdx.x; item < items; item += gridDim.x) {
         const int bin = item / g.n_slices, slice = item - bin * g.n_slices;
@@ -661,16 +678,16 @@ __global__ void __launch_bounds__(kGatherThreads, 1) bspline_bwd_gather_kernel(c
                     S.cell[j] = ok ? ((ix - 4 * bx) | ((iy - 4 * by) << 8) | ((iz - 4 * bz) << 16)) : -1;
                 A wv[EA], wl[EA], wg[3][EA], gt[3][EA];
                 const bool use = ok && o0 < n_orb;
-                load_run<A>(use && gvp ? gvp + ip * n_orb + o0 : nullptr, wv, o0, n_orb, EA);
-                load_run<A>(use && glp ? glp + ip * n_orb + o0 : nullptr, wl, o0, n_orb, EA);
+                load_run<A, EA>(use && gvp ? gvp + ip * n_orb + o0 : nullptr, wv, o0, n_orb, b.vec_up);
+                load_run<A, EA>(use && glp ? glp + ip * n_orb + o0 : nullptr, wl, o0, n_orb, b.vec_up);
 #pragma unroll
                 for (int a = 0; a < 3; ++a)
-                    load_run<A>(use && ggp ? ggp + (ip * 3 + a) * n_orb + o0 : nullptr, wg[a], o0, n_orb, EA);
+                    load_run<A, EA>(use && ggp ? ggp + (ip * 3 + a) * n_orb + o0 : nullptr, wg[a], o0, n_orb, b.vec_up);
 #pragma unroll
                 for (int i = 0; i < 3; ++i)
 #pragma unroll
                     for (int e = 0; e < EA; ++e)
-                        gt[i][e] = (A)p.mg[i] * wg[0][e] + (A)p.mg[3 + i] * wg[1][e] + (A)p.mg[6 + i] * wg[2][e];
+                        gt[i][e] = chain_mg<A>(p, i) * wg[0][e] + chain_mg<A>(p, 3 + i) * wg[1][e] + chain_mg<A>(p, 6 + i) * wg[2][e];
                 auto put = [&](int q, const A* v) {
                     A* d = reinterpret_cast<A*>(&S.up[j][q][lane]);
 #pragma unroll
@@ -773,16 +790,16 @@ int launch_one_kind(const BwdArgs& a, cudaStream_t st)
     const int gpw = 32 >> a.e.lanes_log2;
     const long long groups = a.e.n_pos * a.e.tiles;
     const long long warps = (groups + gpw - 1) / gpw;
-    long long blocks = (warps + kEvalThreads / 32 - 1) / (kEvalThreads / 32);
+    long long blocks = (warps + kBwdThreads / 32 - 1) / (kBwdThreads / 32);
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bspline_bwd_kernel<T, LAPTAB, BLOCH, COEF>,
-                                                                  kEvalThreads, 0);
+                                                                  kBwdThreads, 0);
     if (e != cudaSuccess) return cuda_error(e, "occupancy query");
     if (per_sm < 1) per_sm = 1;
     const long long cap = (long long)sm_count() * per_sm;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    bspline_bwd_kernel<T, LAPTAB, BLOCH, COEF><<<(unsigned)blocks, kEvalThreads, 0, st>>>(a);
+    bspline_bwd_kernel<T, LAPTAB, BLOCH, COEF><<<(unsigned)blocks, kBwdThreads, 0, st>>>(a);
     return cuda_error(cudaGetLastError(), "bspline_bwd_kernel launch");
 }
 
@@ -814,8 +831,9 @@ int launch_gather(const BwdArgs& a, const GatherArgs& g, cudaStream_t st)
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_error(e, "gathered adjoint shared memory");
     const int items = g.n_bins * g.n_slices;
-    const int blocks = items < sm_count() ? items : sm_count();
-    bspline_bwd_gather_kernel<A, LAPTAB><<<blocks > 0 ? blocks : 1, kGatherThreads, smem, st>>>(a, g);
+    const int cap = sm_count() * GatherShape<A>::per_sm;
+    const int blocks = items < cap ? items : cap;
+    bspline_bwd_gather_kernel<A, LAPTAB><<<blocks > 0 ? blocks : 1, GatherShape<A>::threads, smem, st>>>(a, g);
     return cuda_error(cudaGetLastError(), "bspline_bwd_gather_kernel launch");
 }
 
@@ -896,10 +914,10 @@ __global__ void __launch_bounds__(kEvalThreads) five_table_bwd_kernel(const BwdA
             const A* gvp = static_cast<const A*>(b.gv);
             const A* ggp = static_cast<const A*>(b.gg);
             const A* glp = static_cast<const A*>(b.gl);
-            load_run<A>(use && gvp ? gvp + ip * n_orb + o0 : nullptr, up[0], o0, n_orb, E);
+            load_run<A, E>(use && gvp ? gvp + ip * n_orb + o0 : nullptr, up[0], o0, n_orb, b.vec_up);
             for (int a = 0; a < 3; ++a)
-                load_run<A>(use && ggp ? ggp + (ip * 3 + a) * n_orb + o0 : nullptr, up[1 + a], o0, n_orb, E);
-            load_run<A>(use && glp ? glp + ip * n_orb + o0 : nullptr, up[4], o0, n_orb, E);
+                load_run<A, E>(use && ggp ? ggp + (ip * 3 + a) * n_orb + o0 : nullptr, up[1 + a], o0, n_orb, b.vec_up);
+            load_run<A, E>(use && glp ? glp + ip * n_orb + o0 : nullptr, up[4], o0, n_orb, b.vec_up);
         }
         if constexpr (BLOCH) {
             const double uk = __fma_rn(p.kred[0], r[0], __fma_rn(p.kred[1], r[1], __dmul_rn(p.kred[2], r[2])));
@@ -1076,8 +1094,8 @@ __global__ void __launch_bounds__(kEvalThreads) pp_bwd_kernel(const BwdArgs b)
     const size_t colb = (size_t)p.col_stride * sizeof(T);
     const int n_orb = p.n_orb;
     const size_t canon = (size_t)p.nx * p.ny * p.nz * n_orb;
-    const A ml0 = (A)p.ml[0], ml1 = (A)p.ml[1], ml2 = (A)p.ml[2];
-    const A ml3 = (A)p.ml[3], ml4 = (A)p.ml[4], ml5 = (A)p.ml[5];
+    const A ml0 = chain_ml<A>(p, 0), ml1 = chain_ml<A>(p, 1), ml2 = chain_ml<A>(p, 2);
+    const A ml3 = chain_ml<A>(p, 3), ml4 = chain_ml<A>(p, 4), ml5 = chain_ml<A>(p, 5);
 
     for (long long w0 = warp * gpw; w0 < total; w0 += wstride * gpw) {
         const long long gid = w0 + (lane >> p.lanes_log2);
@@ -1104,16 +1122,16 @@ __global__ void __launch_bounds__(kEvalThreads) pp_bwd_kernel(const BwdArgs b)
             const A* gvp = static_cast<const A*>(b.gv);
             const A* ggp = static_cast<const A*>(b.gg);
             const A* glp = static_cast<const A*>(b.gl);
-            load_run<A>(use && gvp ? gvp + ip * n_orb + o0 : nullptr, wv, o0, n_orb, E);
-            load_run<A>(use && glp ? glp + ip * n_orb + o0 : nullptr, wl, o0, n_orb, E);
+            load_run<A, E>(use && gvp ? gvp + ip * n_orb + o0 : nullptr, wv, o0, n_orb, b.vec_up);
+            load_run<A, E>(use && glp ? glp + ip * n_orb + o0 : nullptr, wl, o0, n_orb, b.vec_up);
             for (int a = 0; a < 3; ++a)
-                load_run<A>(use && ggp ? ggp + (ip * 3 + a) * n_orb + o0 : nullptr, wg[a], o0, n_orb, E);
+                load_run<A, E>(use && ggp ? ggp + (ip * 3 + a) * n_orb + o0 : nullptr, wg[a], o0, n_orb, b.vec_up);
             if constexpr (BLOCH) bloch_upstream<A, E, false>(p, r, wv, wg, wl, hv, hg, hl);
 #pragma unroll
             for (int i = 0; i < 3; ++i)
 #pragma unroll
                 for (int e = 0; e < E; ++e)
-                    gt[i][e] = (A)p.mg[i] * wg[0][e] + (A)p.mg[3 + i] * wg[1][e] + (A)p.mg[6 + i] * wg[2][e];
+                    gt[i][e] = chain_mg<A>(p, i) * wg[0][e] + chain_mg<A>(p, 3 + i) * wg[1][e] + chain_mg<A>(p, 6 + i) * wg[2][e];
         }
         int xs[2], ys[2], zs[2];
 #pragma unroll
@@ -1281,6 +1299,8 @@ int launch_bspline_backward(Handle* h, const double* pos, long long n_pos, const
     const size_t ob = (h->storage == QMCSPL_F64 || h->storage == QMCSPL_DF64) ? 8 : 4;
     const uintptr_t al = (uintptr_t)dcoef | (uintptr_t)dcoef_lap;
     a.vec_atomic = ((h->n_orb * ob) % 16 == 0) && (al % 16 == 0);
+    const uintptr_t ul = (uintptr_t)gv | (uintptr_t)gg | (uintptr_t)gl;
+    a.vec_up = ((h->n_orb * ob) % 16 == 0) && (ul % 16 == 0);
     if (dpos) {
         cudaError_t e = cudaMemsetAsync(dpos, 0, sizeof(double) * 3 * (size_t)n_pos, st);
         if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync(dpos)");

@@ -19,14 +19,42 @@ struct BwdArgs {
     void* dcoef_lap;
     double* dpos;             // [P][3], zeroed before the launch, accumulated
     int vec_atomic;           // dcoef rows allow 16-byte vector atomics
+    int vec_up;               // upstream rows allow 16-byte loads
     int bloch;                // complex Bloch outputs: pairs (Re u, Im u) of stored functions (selects the kernel)
 };
 
 namespace {
 
-template <typename A>
-__device__ __forceinline__ void load_run(const A* src, A* v, int o0, int n_orb, int E)
+// The chain-rule constants in the adjoint's type (float: rounded on the host; a conversion from
+// double here is an FP64 instruction, 64 cycles a warp, and a position took nine).
+template <typename A> __device__ __forceinline__ A chain_mg(const EvalArgs& p, int i)
 {
+    if constexpr (sizeof(A) == 4) return p.mgf[i];
+    else return p.mg[i];
+}
+template <typename A> __device__ __forceinline__ A chain_ml(const EvalArgs& p, int i)
+{
+    if constexpr (sizeof(A) == 4) return p.mlf[i];
+    else return p.ml[i];
+}
+
+// E consecutive upstream values of a row (zero past its end, or without a source); vec: whole 16-byte
+// chunks on 16-byte boundaries (BwdArgs::vec_up), read as such: value by value each load instruction
+// would touch all the sectors of the E.
+template <typename A, int E>
+__device__ __forceinline__ void load_run(const A* src, A* v, int o0, int n_orb, int vec)
+{
+    constexpr int C = 16 / sizeof(A);   // values per 16-byte chunk
+    if (vec && src && o0 + E <= n_orb) {
+#pragma unroll
+        for (int j = 0; j < E; j += C) {
+            const uint4 r = __ldg(reinterpret_cast<const uint4*>(src + j));
+            if constexpr (C == 4) unpack<float>(r, v + j);
+            else unpack<double>(r, v + j);
+        }
+        return;
+    }
+#pragma unroll
     for (int j = 0; j < E; ++j) v[j] = (src && o0 + j < n_orb) ? src[j] : A(0);
 }
 
@@ -110,8 +138,8 @@ __device__ __forceinline__ double bloch_phase_sum(const EvalArgs& p, const A* u0
 {
     const A ka[3] = {(A)p.kc[0], (A)p.kc[1], (A)p.kc[2]};
     const A kk = ka[0] * ka[0] + ka[1] * ka[1] + ka[2] * ka[2];
-    const A ml0 = (A)p.ml[0], ml1 = (A)p.ml[1], ml2 = (A)p.ml[2];
-    const A ml3 = (A)p.ml[3], ml4 = (A)p.ml[4], ml5 = (A)p.ml[5];
+    const A ml0 = chain_ml<A>(p, 0), ml1 = chain_ml<A>(p, 1), ml2 = chain_ml<A>(p, 2);
+    const A ml3 = chain_ml<A>(p, 3), ml4 = chain_ml<A>(p, 4), ml5 = chain_ml<A>(p, 5);
     auto imc = [](A hr, A hi, A wr, A wi) { return hr * wi - hi * wr; };   // Im(conj(h) w)
     double sph = 0.0;
 #pragma unroll
@@ -120,8 +148,8 @@ __device__ __forceinline__ double bloch_phase_sum(const EvalArgs& p, const A* u0
         A gc[3][2];   // Cartesian gradient of Re u, Im u
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            gc[a][0] = (A)p.mg[3 * a] * g1[0][r] + (A)p.mg[3 * a + 1] * g1[1][r] + (A)p.mg[3 * a + 2] * g1[2][r];
-            gc[a][1] = (A)p.mg[3 * a] * g1[0][q] + (A)p.mg[3 * a + 1] * g1[1][q] + (A)p.mg[3 * a + 2] * g1[2][q];
+            gc[a][0] = chain_mg<A>(p, 3 * a) * g1[0][r] + chain_mg<A>(p, 3 * a + 1) * g1[1][r] + chain_mg<A>(p, 3 * a + 2) * g1[2][r];
+            gc[a][1] = chain_mg<A>(p, 3 * a) * g1[0][q] + chain_mg<A>(p, 3 * a + 1) * g1[1][q] + chain_mg<A>(p, 3 * a + 2) * g1[2][q];
         }
         const A ur = u0[r], ui = u0[q];
         A acc = imc(hv[r], hv[q], ur, ui);

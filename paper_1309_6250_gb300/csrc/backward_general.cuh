@@ -41,8 +41,8 @@ __global__ void __launch_bounds__(kEvalThreads) general_bwd_kernel(const BwdArgs
     const size_t rowb = (size_t)p.row_stride * sizeof(T);
     const size_t colb = (size_t)p.col_stride * sizeof(T);
     const int n_orb = p.n_orb;
-    const A ml0 = (A)p.ml[0], ml1 = (A)p.ml[1], ml2 = (A)p.ml[2];
-    const A ml3 = (A)p.ml[3], ml4 = (A)p.ml[4], ml5 = (A)p.ml[5];
+    const A ml0 = chain_ml<A>(p, 0), ml1 = chain_ml<A>(p, 1), ml2 = chain_ml<A>(p, 2);
+    const A ml3 = chain_ml<A>(p, 3), ml4 = chain_ml<A>(p, 4), ml5 = chain_ml<A>(p, 5);
 
     for (long long w0 = warp * gpw; w0 < total; w0 += wstride * gpw) {
         const long long gid = w0 + (lane >> p.lanes_log2);
@@ -97,16 +97,16 @@ __global__ void __launch_bounds__(kEvalThreads) general_bwd_kernel(const BwdArgs
             const A* ggp = static_cast<const A*>(b.gg);
             const A* glp = static_cast<const A*>(b.gl);
             const bool use = active && ok && o0 < n_orb;
-            load_run<A>(use && gvp ? gvp + ip * n_orb + o0 : nullptr, wv, o0, n_orb, E);
-            load_run<A>(use && glp ? glp + ip * n_orb + o0 : nullptr, wl, o0, n_orb, E);
+            load_run<A, E>(use && gvp ? gvp + ip * n_orb + o0 : nullptr, wv, o0, n_orb, b.vec_up);
+            load_run<A, E>(use && glp ? glp + ip * n_orb + o0 : nullptr, wl, o0, n_orb, b.vec_up);
             for (int a = 0; a < 3; ++a)
-                load_run<A>(use && ggp ? ggp + (ip * 3 + a) * n_orb + o0 : nullptr, wg[a], o0, n_orb, E);
+                load_run<A, E>(use && ggp ? ggp + (ip * 3 + a) * n_orb + o0 : nullptr, wg[a], o0, n_orb, b.vec_up);
             if constexpr (BLOCH) bloch_upstream<A, E, LAPTAB>(p, p.pos + 3 * ip, wv, wg, wl, hv, hg, hl);
 #pragma unroll
             for (int i = 0; i < 3; ++i)
 #pragma unroll
                 for (int e = 0; e < E; ++e)
-                    gt[i][e] = (A)p.mg[i] * wg[0][e] + (A)p.mg[3 + i] * wg[1][e] + (A)p.mg[6 + i] * wg[2][e];
+                    gt[i][e] = chain_mg<A>(p, i) * wg[0][e] + chain_mg<A>(p, 3 + i) * wg[1][e] + chain_mg<A>(p, 6 + i) * wg[2][e];
         }
 
         // ---- coefficient adjoint: scatter into the W^3 stencil rows ----
