@@ -549,6 +549,120 @@ __global__ void __launch_bounds__(32, kSmallWarps) bspline_vgl_small_kernel(cons
     warp_task<T, LAPTAB, kSmallAhead, RAGGED>(p, w0, threadIdx.x, stage);
 }
 
+// ---- small launches of FP64 tables: one orbital per lane, shared column weights ----
+// The FP64 pipe takes a warp instruction every 64 cycles per SM sub-partition, so a small launch
+// lasts as long as one warp's instructions: 907 per lane above with the Hessian Laplacian and two
+// orbitals, a third of them weights that every lane of a position computes alike.  Here a lane takes
+// one orbital (twice the lanes per position, on sub-partitions that were idle) and the lanes of a
+// position divide the three axes' weights and the 16 columns' among themselves, through shared
+// memory: the same products and sums in the same order, about 410 instructions.  1,000 positions x 8
+// orbitals with the Hessian Laplacian: 33 -> 16 us (127 us in blocks of 16 warps).
+struct F64Shared {
+    double axis[8][3][12];    // per group (at most 8: groups of at least 4 lanes): w, dw, d2w of each axis
+    double col[8][16][6];     // w00, w10, w01, c0, c1, c2 of each stencil column
+};
+
+template <bool LAPTAB>
+__device__ __forceinline__ void bspline_warp_task_f64_lanes(const EvalArgs& p, long long w0, int lane, F64Shared& sh)
+{
+    const int L = 1 << p.lanes_log2;          // at least 4
+    const int sub = lane & (L - 1);
+    const int gbase = lane & ~(L - 1);
+    const int grp = lane >> p.lanes_log2;
+    const size_t rowb = (size_t)p.row_stride * 8;
+    const size_t colb = (size_t)p.col_stride * 8;
+    const long long gid = w0 + grp;
+    const bool active = gid < p.n_pos * p.tiles;
+    const long long q = active ? gid / p.tiles : 0;
+    const int tile = active ? (int)(gid - q * p.tiles) : 0;
+    const long long ip = active ? order_index(p, q) : 0;
+    int ix, iy, iz;
+    double tx, ty, tz;
+    bool ok;
+    coords_double(p, ip, L, sub, gbase, ix, iy, iz, tx, ty, tz, ok);
+    if (active && !ok && sub == 0 && tile == 0) atomicOr(p.err, 1);
+    if (sub < 3) {   // one axis per lane
+        double w[4], dw[4], d2w[4];
+        bspline_weights<double>(sub == 0 ? tx : sub == 1 ? ty : tz, w, dw, LAPTAB ? nullptr : d2w);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            sh.axis[grp][sub][j] = w[j];
+            sh.axis[grp][sub][4 + j] = dw[j];
+            if (!LAPTAB) sh.axis[grp][sub][8 + j] = d2w[j];
+        }
+    }
+    __syncwarp();
+    const double *ax = sh.axis[grp][0], *ay = sh.axis[grp][1], *az = sh.axis[grp][2];
+    for (int c = sub; c < 16; c += L) {
+        const int l = c >> 2, m = c & 3;
+        const double bx = ax[l], dbx = ax[4 + l], by = ay[m], dby = ay[4 + m];
+        const double w00 = bx * by, w10 = dbx * by, w01 = bx * dby;
+        sh.col[grp][c][0] = w00;
+        sh.col[grp][c][1] = w10;
+        sh.col[grp][c][2] = w01;
+        if (!LAPTAB) {
+            const double d2bx = ax[8 + l], d2by = ay[8 + m];
+            sh.col[grp][c][3] = p.ml[0] * (d2bx * by) + p.ml[1] * (bx * d2by) + p.ml[3] * (dbx * dby);
+            sh.col[grp][c][4] = p.ml[4] * w10 + p.ml[5] * w01;
+            sh.col[grp][c][5] = p.ml[2] * w00;
+        }
+    }
+    __syncwarp();
+    const int o = tile * L + sub;             // this lane's orbital
+    if (!active || o >= p.n_orb) return;
+    double bz[4], dbz[4], d2bz[4];
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+        bz[n] = az[n];
+        dbz[n] = az[4 + n];
+        if (!LAPTAB) d2bz[n] = az[8 + n];
+    }
+    int xs[4], ys[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        xs[j] = wrap1(ix + j - 1, p.nx);
+        ys[j] = wrap1(iy + j - 1, p.ny);
+    }
+    const char* t0 = static_cast<const char*>(p.tab[0]) + (size_t)o * 8 + (size_t)iz * rowb;
+    const char* t1 = LAPTAB ? static_cast<const char*>(p.tab[1]) + (size_t)o * 8 + (size_t)iz * rowb : nullptr;
+    double v = 0.0, gx = 0.0, gy = 0.0, gz = 0.0, lp = 0.0;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+        const size_t col = (size_t)(xs[c >> 2] * p.ny + ys[c & 3]) * colb;
+        double a0 = 0.0, a1 = 0.0, a2 = 0.0, al = 0.0;
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            const double t = ldg_table8(p, t0 + col + n * rowb);
+            a0 = fma(bz[n], t, a0);
+            a1 = fma(dbz[n], t, a1);
+            if (!LAPTAB) a2 = fma(d2bz[n], t, a2);
+            else al = fma(bz[n], ldg_table8(p, t1 + col + n * rowb), al);
+        }
+        const double* w = sh.col[grp][c];
+        v = fma(w[0], a0, v);
+        gx = fma(w[1], a0, gx);
+        gy = fma(w[2], a0, gy);
+        gz = fma(w[0], a1, gz);
+        if (LAPTAB) lp = fma(w[0], al, lp);
+        else lp = fma(w[3], a0, fma(w[4], a1, fma(w[5], a2, lp)));
+    }
+    const long long row = ip * p.n_orb + o;
+    if (p.val) __stcs(static_cast<double*>(p.val) + row, v);
+    if (p.grad)
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            __stcs(static_cast<double*>(p.grad) + row + (2 * ip + a) * p.n_orb,
+                   fma(p.mg[3 * a], gx, fma(p.mg[3 * a + 1], gy, p.mg[3 * a + 2] * gz)));
+    if (p.lap) __stcs(static_cast<double*>(p.lap) + row, lp);
+}
+
+template <bool LAPTAB>
+__global__ void __launch_bounds__(32) bspline_vgl_f64_lanes_kernel(const EvalArgs p)
+{
+    __shared__ F64Shared sh;
+    bspline_warp_task_f64_lanes<LAPTAB>(p, (long long)blockIdx.x << (5 - p.lanes_log2), threadIdx.x, sh);
+}
+
 // Several cells in one launch: warp task w belongs to the cell c with
 // start[c] <= w < start[c + 1]; tasks are handed out round-robin over all warps.
 struct BatchArgs {
@@ -602,6 +716,19 @@ int launch_shape(const EvalArgs& a, long long warps, cudaStream_t st)
 template <typename T, bool LAPTAB>
 int launch_small(const EvalArgs& a, long long warps, cudaStream_t st)
 {
+    if constexpr (std::is_same<T, double>::value) {
+        // one orbital per lane while that leaves at most a warp per sub-partition of every SM: beyond, the
+        // FP64 pipes are busy either way and the weights are better shared by two orbitals.  (Groups of
+        // four lanes or more, for the shared weights; Bloch orbitals need Re and Im in one lane.)
+        EvalArgs b = a;
+        if (b.lanes_log2 < 5) ++b.lanes_log2;
+        else b.tiles *= 2;
+        const long long gpw = 32 >> b.lanes_log2, w = (b.n_pos * b.tiles + gpw - 1) / gpw;
+        if (b.lanes_log2 >= 2 && !b.phase && w <= 4LL * sm_count()) {
+            bspline_vgl_f64_lanes_kernel<LAPTAB><<<(unsigned)w, 32, 0, st>>>(b);
+            return cuda_error(cudaGetLastError(), "bspline_vgl_f64_lanes_kernel launch");
+        }
+    }
     auto k = bspline_vgl_small_kernel<T, LAPTAB, false>;
     if constexpr (kStaged<T>) {
         if (!a.vec_out) k = bspline_vgl_small_kernel<T, LAPTAB, true>;

@@ -40,6 +40,18 @@ __device__ __forceinline__ uint4 ldg_table(const EvalArgs& p, const char* a)
     return ldg16(a);
 }
 
+// One double of a table, checked likewise.
+__device__ __forceinline__ double ldg_table8(const EvalArgs& p, const char* a)
+{
+#ifdef QMCSPL_DEBUG_BOUNDS
+    if (a < p.tab_lo || a + 8 > p.tab_hi || (reinterpret_cast<uintptr_t>(a) & 7)) {
+        atomicOr(p.err, 2);
+        return 0.0;
+    }
+#endif
+    return __ldg(reinterpret_cast<const double*>(a));
+}
+
 // The position evaluated q-th (through the evaluation order when there is one); range
 // checked in QMCSPL_DEBUG_BOUNDS builds (bit 1 of the error word, position 0 used instead).
 __device__ __forceinline__ long long order_index(const EvalArgs& p, long long q)
