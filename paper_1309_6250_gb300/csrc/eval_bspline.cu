@@ -163,7 +163,8 @@ __device__ __forceinline__ void bspline_warp_task(const EvalArgs& p, long long w
 // (fma.rn.f32x2: two orbitals per instruction) and the rows of the next AHEAD stencil columns
 // loaded before the current column is contracted.
 // stage: with RAGGED, the warp's shared memory for the stores of unaligned rows (see RaggedStore).
-template <typename T, bool LAPTAB, int AHEAD, bool RAGGED>
+// NOREC: for launches without records (coords_float_shared).
+template <typename T, bool LAPTAB, int AHEAD, bool RAGGED, bool NOREC>
 __device__ __forceinline__ void bspline_warp_task_x2(const EvalArgs& p, long long w0, int lane, float* stage)
 {
     constexpr int E = Traits<T>::E;          // orbitals per lane (4 float, 8 bfloat16)
@@ -186,7 +187,8 @@ __device__ __forceinline__ void bspline_warp_task_x2(const EvalArgs& p, long lon
     bool ok;
     // (the bfloat16 kernel runs fastest with the rolled form of the reduction, the float one with
     // the written-out form; both give the same bits)
-    coords_float<std::is_same<T, __nv_bfloat16>::value>(p, ip, L, sub, gbase, ix, iy, iz, tx, ty, tz, ok);
+    if constexpr (NOREC) coords_float_shared(p, ip, L, sub, gbase, ix, iy, iz, tx, ty, tz, ok);
+    else coords_float<std::is_same<T, __nv_bfloat16>::value>(p, ip, L, sub, gbase, ix, iy, iz, tx, ty, tz, ok);
     if (!RAGGED && !active) return;   // (all lanes take part in the staged stores)
     if (active && !ok && sub == 0 && tile == 0) atomicOr(p.err, 1);
 
@@ -492,12 +494,12 @@ __device__ __forceinline__ void bspline_warp_task_df(const EvalArgs& p, long lon
 
 // float and bfloat16 tables take the packed path, double tables the scalar one.  AHEAD: columns of
 // rows in flight (packed path; columns unrolled for double-float tables).
-template <typename T, bool LAPTAB, int AHEAD = 1, bool RAGGED = false>
+template <typename T, bool LAPTAB, int AHEAD = 1, bool RAGGED = false, bool NOREC = false>
 __device__ __forceinline__ void warp_task(const EvalArgs& p, long long w0, int lane, float* stage = nullptr)
 {
     if constexpr (std::is_same<T, DF64Tag>::value) bspline_warp_task_df<LAPTAB, AHEAD>(p, w0, lane);
     else if constexpr (sizeof(T) == 8) bspline_warp_task<T, LAPTAB>(p, w0, lane);
-    else bspline_warp_task_x2<T, LAPTAB, AHEAD, RAGGED>(p, w0, lane, stage);
+    else bspline_warp_task_x2<T, LAPTAB, AHEAD, RAGGED, NOREC>(p, w0, lane, stage);
 }
 
 #ifndef QMCSPL_EVAL_THREADS
@@ -523,7 +525,7 @@ template <> struct BspBlock<float, true> {
 };
 constexpr int kLargeLaunchRounds = 4;   // warp-task rounds from which the large shape is used
 
-template <typename T, bool LAPTAB, int THREADS, bool RAGGED>
+template <typename T, bool LAPTAB, int THREADS, bool RAGGED, bool NOREC = false>
 __global__ void __launch_bounds__(THREADS, 1) bspline_vgl_kernel(const EvalArgs p)
 {
     constexpr int WPB = THREADS / 32;
@@ -534,19 +536,19 @@ __global__ void __launch_bounds__(THREADS, 1) bspline_vgl_kernel(const EvalArgs 
     const long long warp = (long long)blockIdx.x * WPB + (threadIdx.x >> 5);
     const long long wstride = (long long)gridDim.x * WPB;
     for (long long w0 = warp * gpw; w0 < total; w0 += wstride * gpw)
-        warp_task<T, LAPTAB, 1, RAGGED>(p, w0, lane, stage[RAGGED ? threadIdx.x >> 5 : 0]);
+        warp_task<T, LAPTAB, 1, RAGGED, NOREC>(p, w0, lane, stage[RAGGED ? threadIdx.x >> 5 : 0]);
 }
 
 // Launches of at most kSmallWarps warp tasks per SM: a block per warp task, so that they spread over
 // all SMs, and three columns of rows in flight (the registers of the missing warps are free), since
 // nothing but a warp's own loads hides their latency.
 constexpr int kSmallAhead = 3;
-template <typename T, bool LAPTAB, bool RAGGED>
+template <typename T, bool LAPTAB, bool RAGGED, bool NOREC = false>
 __global__ void __launch_bounds__(32, kSmallWarps) bspline_vgl_small_kernel(const EvalArgs p)
 {
     __shared__ __align__(16) float stage[kStageFloats<T, RAGGED>];
     const long long w0 = (long long)blockIdx.x << (5 - p.lanes_log2);
-    warp_task<T, LAPTAB, kSmallAhead, RAGGED>(p, w0, threadIdx.x, stage);
+    warp_task<T, LAPTAB, kSmallAhead, RAGGED, NOREC>(p, w0, threadIdx.x, stage);
 }
 
 // ---- small launches of FP64 tables: one orbital per lane, shared column weights ----
@@ -708,6 +710,9 @@ int launch_shape(const EvalArgs& a, long long warps, cudaStream_t st)
     auto k = bspline_vgl_kernel<T, LAPTAB, THREADS, false>;
     if constexpr (kStaged<T>) {
         if (!a.vec_out) k = bspline_vgl_kernel<T, LAPTAB, THREADS, true>;
+        if constexpr (THREADS == QMCSPL_EVAL_THREADS) {   // (the large shape's launches have records)
+            if (!a.rec) k = a.vec_out ? bspline_vgl_kernel<T, LAPTAB, THREADS, false, true> : bspline_vgl_kernel<T, LAPTAB, THREADS, true, true>;
+        }
     }
     k<<<(unsigned)grid_for(k, THREADS, warps), THREADS, 0, st>>>(a);
     return cuda_error(cudaGetLastError(), "bspline_vgl_kernel launch");
@@ -731,7 +736,8 @@ int launch_small(const EvalArgs& a, long long warps, cudaStream_t st)
     }
     auto k = bspline_vgl_small_kernel<T, LAPTAB, false>;
     if constexpr (kStaged<T>) {
-        if (!a.vec_out) k = bspline_vgl_small_kernel<T, LAPTAB, true>;
+        if (!a.vec_out) k = a.rec ? bspline_vgl_small_kernel<T, LAPTAB, true> : bspline_vgl_small_kernel<T, LAPTAB, true, true>;
+        else if (!a.rec) k = bspline_vgl_small_kernel<T, LAPTAB, false, true>;
     }
     k<<<(unsigned)warps, 32, 0, st>>>(a);
     return cuda_error(cudaGetLastError(), "bspline_vgl_small_kernel launch");

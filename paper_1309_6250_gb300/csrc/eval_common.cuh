@@ -498,6 +498,62 @@ __device__ __forceinline__ void reduced_coordinates_df(const EvalArgs& p, const 
     }
 }
 
+// The same reduction for kernels of launches without records, with the double-to-pair conversions
+// divided among the lanes: a conversion is four FP64 instructions, each 64 cycles of a warp's
+// sub-partition, and with every lane converting the position and its row of a^-1 a task spent 24 of
+// them before its first load (a position of 128 orbitals: 1,500 of some 8,000 cycles).  Here lane j < 9
+// converts a^-1's entry j, and lane j < 3 of a group component j of its position; shuffles hand them
+// round.  Same values, same steps, same bits.  4,096 positions x 128 orbitals in input order: 27.8 -> 24.9 us
+// with the Laplacian table, 18.5 -> 14.0 us without; 8,191 x 40: 30.9 -> 22.2 us.
+__device__ __forceinline__ void coords_float_shared(const EvalArgs& p, long long ip, int L, int sub, int gbase, int& ix,
+                                                    int& iy, int& iz, float& tx, float& ty, float& tz, bool& ok)
+{
+    const int lane = threadIdx.x & 31;
+    const dfloat a = df_from_double(p.ainv[lane < 9 ? lane : 8]);
+    const double* pos = p.pos + 3 * ip;
+    if (L >= 4) {
+        const int ax = sub < 3 ? sub : 2;
+        const dfloat x = df_from_double(pos[ax]);
+        float rh[3], rl[3], ah[3], al[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            rh[j] = __shfl_sync(kFullMask, x.h, gbase + j);
+            rl[j] = __shfl_sync(kFullMask, x.l, gbase + j);
+            ah[j] = __shfl_sync(kFullMask, a.h, 3 * ax + j);
+            al[j] = __shfl_sync(kFullMask, a.l, 3 * ax + j);
+        }
+        const double r[3] = {pos[0], pos[1], pos[2]};   // (for positions far outside the cell)
+        const double* ad = p.ainv + 3 * ax;
+        int i;
+        float t;
+        bool o;
+        reduce_axis_df(r, rh, rl, ad, ah, al, ax == 0 ? p.nx : (ax == 1 ? p.ny : p.nz), i, t, o);
+        ix = __shfl_sync(kFullMask, i, gbase);
+        iy = __shfl_sync(kFullMask, i, gbase + 1);
+        iz = __shfl_sync(kFullMask, i, gbase + 2);
+        tx = __shfl_sync(kFullMask, t, gbase);
+        ty = __shfl_sync(kFullMask, t, gbase + 1);
+        tz = __shfl_sync(kFullMask, t, gbase + 2);
+        const int okb = o ? 1 : 0;
+        ok = (__shfl_sync(kFullMask, okb, gbase) & __shfl_sync(kFullMask, okb, gbase + 1) &
+              __shfl_sync(kFullMask, okb, gbase + 2)) != 0;
+        return;
+    }
+    const double r[3] = {pos[0], pos[1], pos[2]};
+    float rh[3], rl[3], ah[9], al[9];
+    df_row(r, rh, rl);
+#pragma unroll
+    for (int j = 0; j < 9; ++j) {
+        ah[j] = __shfl_sync(kFullMask, a.h, j);
+        al[j] = __shfl_sync(kFullMask, a.l, j);
+    }
+    bool o0, o1, o2;
+    reduce_axis_df(r, rh, rl, p.ainv, ah, al, p.nx, ix, tx, o0);
+    reduce_axis_df(r, rh, rl, p.ainv + 3, ah + 3, al + 3, p.ny, iy, ty, o1);
+    reduce_axis_df(r, rh, rl, p.ainv + 6, ah + 6, al + 6, p.nz, iz, tz, o2);
+    ok = o0 && o1 && o2;
+}
+
 // Cubic B-spline weights (Eq. b-splinebasis) and first derivatives in double-float
 // from a reduced coordinate given in double.
 __device__ __forceinline__ void bspline_weights_df(dfloat t, dfloat* w, dfloat* dw, dfloat* d2w)
