@@ -23,7 +23,8 @@
 // error-free FP32 multiply-add done two columns at a time with fma.rn.f32x2 (see df_fma2):
 // the FP32 pipe carries it, several times faster on this part.  Every loop is bounded by n.
 // Complex orbitals (Bloch functions) take a complex elimination, in FP64 (slater_complex_kernel)
-// or in double-float (slater_cdf_kernel).
+// or in double-float (slater_cdf_kernel).  The double-float kernels here serve the largest spin blocks;
+// smaller ones keep their matrix in registers (slater_reg.cu, slater_creg.cu).
 #include <cmath>
 
 #include "slater_common.cuh"
@@ -454,12 +455,7 @@ __global__ void __launch_bounds__(NT) slater_df_kernel(const SlaterArgs a)
 // ln|det A| = sum_k ln|d_k| and the phase of det A is sum_k arg d_k + pi (number of row swaps),
 // reported as (cos, sin).  The kinetic term and the drift are complex (Jacobi's formula).
 constexpr int kSlaterCplxMaxBlock = QMCSPL_SLATER_MAX_COMPLEX_BLOCK;
-// complex double-float kernel: blocks small enough for two CTAs per SM in shared memory run
-// 256-thread CTAs, two per SM, so that one walker's barriers and pivot search overlap the
-// other's updates (64 + 64 electrons: 15.5 -> 10.2 ms for 4,096 walkers); larger blocks run one
-// 512-thread CTA per SM
-constexpr int kSlaterCdfThreadsSmall = 256;
-constexpr int kSlaterCdfThreadsLarge = 512;
+constexpr int kSlaterCdfThreads = 512;   // complex double-float kernel: one CTA per SM, as above
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b)
 {
@@ -654,13 +650,14 @@ __global__ void __launch_bounds__(kSlaterThreads) slater_complex_kernel(const Sl
     }
 }
 
-// Complex entries in double-float: four float arrays Rh, Rl, Ih, Il of [n][ns] (real and
-// imaginary parts, each a pair h + l), ns = n rounded up to even, plus 2, as in
+// Complex entries in double-float, for spin blocks of more than kSlaterCregMaxBlock electrons
+// (smaller ones: slater_creg.cu, the matrix in registers): four float arrays Rh, Rl, Ih, Il of
+// [n][ns] (real and imaginary parts, each a pair h + l), ns = n rounded up to even, plus 2, as in
 // slater_df_kernel.  The update A[i][j] -= f_i r_j of a complex multiplier f and row entry r is
 // four error-free packed multiply-adds (re += (-f.re) r.re + f.im r.im, im += (-f.re) r.im +
 // (-f.im) r.re), renormalised; 1/d = conj(d) / |d|^2 with the double-float reciprocal.
 template <typename T, int NT>
-__global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) slater_cdf_kernel(const SlaterArgs a)
+__global__ void __launch_bounds__(NT) slater_cdf_kernel(const SlaterArgs a)
 {
     extern __shared__ float csf[];
     __shared__ double red[NT / 32];
@@ -940,15 +937,14 @@ template <typename T>
 int launch_slater_complex(const SlaterArgs& a, int nmax, cudaStream_t st)
 {
     if (a.arith == 1) {
+        if (nmax <= kSlaterCregMaxBlock)
+            return sizeof(T) == 8 ? launch_slater_creg_f64(a, nmax, st) : launch_slater_creg_f32(a, nmax, st);
         const int ns = ((nmax + 1) & ~1) + 2;
         const size_t smem = 4 * (size_t)nmax * ns * sizeof(float);
-        // static shared memory of the kernel is under 11 KB; 227 KB per SM
-        const bool two = 2 * (smem + 11 * 1024) <= 227 * 1024;
-        auto k = two ? slater_cdf_kernel<T, kSlaterCdfThreadsSmall> : slater_cdf_kernel<T, kSlaterCdfThreadsLarge>;
-        const int nt = two ? kSlaterCdfThreadsSmall : kSlaterCdfThreadsLarge;
+        auto k = slater_cdf_kernel<T, kSlaterCdfThreads>;
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute(slater_cdf_kernel)");
-        k<<<(unsigned)a.n_walkers, nt, smem, st>>>(a);
+        k<<<(unsigned)a.n_walkers, kSlaterCdfThreads, smem, st>>>(a);
         return cuda_error(cudaGetLastError(), "slater_cdf_kernel launch");
     }
     const size_t smem = (size_t)nmax * (nmax + 1) * sizeof(double2);

@@ -50,103 +50,6 @@ template <> struct RegShape<2> { static constexpr int RL = 2, CP = 8, NW = 4, pe
 template <> struct RegShape<3> { static constexpr int RL = 3, CP = 6, NW = 8, per_sm = 2; };
 template <> struct RegShape<4> { static constexpr int RL = 4, CP = 4, NW = 16, per_sm = 1; };
 
-// (h, l) <- h + l with |l| <= ulp(h) / 2.  Three operations do what the full two-sum does: h is a
-// sum whose terms cancel only to a multiple of their last place, so it is 0 or no smaller than about l.
-__device__ __forceinline__ void quick_norm2(f32x2& h, f32x2& l)
-{
-    const f32x2 s = add2(h, l);
-    l = sub2(l, sub2(s, h));
-    h = s;
-}
-
-// (H, L) -= f r for a row's multiplier f = (fh, fh), (fl, fl) and a column pair of the pivot row as
-// (rh0, rh1), its negative and the negative of (rl0, rl1): df_fma2's steps and a renormalisation
-// (entries are updated n times and reused as pivots, multipliers and reciprocals, which assume
-// |lo| << |hi|).
-__device__ __forceinline__ void eliminate2(f32x2& H, f32x2& L, f32x2 fh, f32x2 fl, f32x2 rh, f32x2 nrh, f32x2 nrl)
-{
-    const f32x2 P = mul2(fh, rh);
-    f32x2 E = ffma2(fh, nrh, P);
-    E = ffma2(fh, nrl, E);
-    E = ffma2(fl, nrh, E);
-    const f32x2 S = sub2(H, P);
-    const f32x2 BB = sub2(S, H);
-    const f32x2 T1 = sub2(H, sub2(S, BB));
-    const f32x2 T2 = add2(P, BB);
-    L = add2(L, add2(sub2(T1, T2), E));
-    H = S;
-    quick_norm2(H, L);
-}
-
-// (H, L) += x y for double-float x = xh + xl and y = yh + yl (yl only where WIDE): df_fma2's steps
-template <bool WIDE>
-__device__ __forceinline__ void dot2(f32x2& H, f32x2& L, f32x2 xh, f32x2 nxh, f32x2 xl, f32x2 yh, f32x2 yl)
-{
-    const f32x2 nP = mul2(nxh, yh);
-    f32x2 E = ffma2(xh, yh, nP);
-    if (WIDE) E = ffma2(xh, yl, E);
-    E = ffma2(xl, yh, E);
-    const f32x2 S = sub2(H, nP);
-    const f32x2 B = sub2(S, H);
-    const f32x2 T1 = sub2(H, sub2(S, B));
-    const f32x2 T2 = add2(nP, B);
-    L = add2(L, add2(sub2(T1, T2), E));
-    H = S;
-}
-
-// sum over the warp of double-float pairs; every lane gets the total
-__device__ __forceinline__ void warp_sum2(f32x2& H, f32x2& L)
-{
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const f32x2 h = __shfl_xor_sync(kFullMask, H, off), l = __shfl_xor_sync(kFullMask, L, off);
-        const f32x2 S = add2(H, h);
-        const f32x2 BB = sub2(S, H);
-        const f32x2 T = add2(sub2(H, sub2(S, BB)), sub2(h, BB));
-        L = add2(T, add2(L, l));
-        H = S;
-        quick_norm2(H, L);
-    }
-}
-
-__device__ __forceinline__ void split(float v, float& h, float& l)
-{
-    h = v;
-    l = 0.0f;
-}
-__device__ __forceinline__ void split(double v, float& h, float& l)
-{
-    const dfloat d = df_from_double(v);
-    h = d.h;
-    l = d.l;
-}
-
-// ---- mbarriers (one arrival each, never reused) ----
-__device__ __forceinline__ void mbar_init(uint64_t* bar)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(bar)) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((unsigned)__cvta_generic_to_shared(bar)) : "memory");
-}
-// Waits for the arrival, about a second at most: false if it did not come.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar)
-{
-    const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
-    long long t0 = 0;
-    for (int i = 0;; ++i) {
-        unsigned done;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done)
-                     : "r"(a)
-                     : "memory");
-        if (done) return true;
-        if (i == 0) t0 = clock64();
-        else if (clock64() - t0 > (1LL << 31)) return false;
-    }
-}
-
 struct BlockResult {
     double logdet, kin;
     int odd;         // determinant negative
