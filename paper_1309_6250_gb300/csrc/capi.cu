@@ -111,13 +111,13 @@ void fill_eval_args(const Handle* h, EvalArgs* a)
     std::memcpy(a->ml, h->ml, sizeof(a->ml));
     for (int i = 0; i < 9; ++i) {
         a->mgf[i] = (float)h->mg[i];
-        a->mgh[i] = (float)h->mg[i];
-        a->mgl[i] = (float)(h->mg[i] - (double)a->mgh[i]);
+        a->mgl[i] = (float)(h->mg[i] - (double)a->mgf[i]);
+        a->ainvh[i] = (float)h->ainv[i];
+        a->ainvl[i] = (float)(h->ainv[i] - (double)a->ainvh[i]);
     }
     for (int i = 0; i < 6; ++i) {
         a->mlf[i] = (float)h->ml[i];
-        a->mlh[i] = (float)h->ml[i];
-        a->mll[i] = (float)(h->ml[i] - (double)a->mlh[i]);
+        a->mll[i] = (float)(h->ml[i] - (double)a->mlf[i]);
     }
     a->err = h->d_err;
     a->tab_lo = static_cast<const char*>(h->tables);
@@ -542,7 +542,7 @@ static int eval_dispatch(Handle* h, const double* pos, long long n_pos, void* va
     }
     const bool sort = use_cell_order(h, n_pos);
     // Bloch handles always take the per-position pass: it computes the phase factors
-    if (sort || n_pos >= kRecordMinPositions || h->bloch) {
+    if (sort || h->bloch || (n_pos >= kRecordMinPositions && !eval_shares_coordinates(h, n_pos))) {
         const int rc = prepare_positions(h, pos, n_pos, sort, &pr, st);
         if (rc != QMCSPL_OK) return rc;
     }

@@ -366,7 +366,7 @@ __device__ __forceinline__ void bspline_warp_task_df(const EvalArgs& p, long lon
     dfloat ml[6];
     if (!LAPTAB)
 #pragma unroll
-        for (int k = 0; k < 6; ++k) ml[k] = {p.mlh[k], p.mll[k]};
+        for (int k = 0; k < 6; ++k) ml[k] = {p.mlf[k], p.mll[k]};
     int xs[4], ys[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -449,7 +449,7 @@ __device__ __forceinline__ void bspline_warp_task_df(const EvalArgs& p, long lon
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             f32x2 Gh = 0, Gl = 0;
-            const float m0h = p.mgh[3 * a], m1h = p.mgh[3 * a + 1], m2h = p.mgh[3 * a + 2];
+            const float m0h = p.mgf[3 * a], m1h = p.mgf[3 * a + 1], m2h = p.mgf[3 * a + 2];
             const float m0l = p.mgl[3 * a], m1l = p.mgl[3 * a + 1], m2l = p.mgl[3 * a + 2];
             df_mad2(Gh, Gl, pack2(m0h, m0h), pack2(m0l, m0l), Xh, Xl, zero);
             df_mad2(Gh, Gl, pack2(m1h, m1h), pack2(m1l, m1l), Yh, Yl, zero);
@@ -672,7 +672,7 @@ struct BatchArgs {
     long long start[QMCSPL_MAX_BATCH + 1];   // prefix sums of warp tasks per cell
     EvalArgs cell[QMCSPL_MAX_BATCH];
 };
-static_assert(sizeof(BatchArgs) <= 32000, "batched kernel parameters exceed the 32 KB limit");
+static_assert(sizeof(BatchArgs) <= 32764, "batched kernel parameters exceed the limit");
 
 template <typename T, bool LAPTAB, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) bspline_vgl_batched_kernel(const __grid_constant__ BatchArgs b)
@@ -795,6 +795,23 @@ void set_outputs(const Handle* h, EvalArgs& a, void* val, void* grad, void* lap)
 }
 
 }  // namespace
+
+// Float and bfloat16 cubic tables, launches below the large shape: the kernels without records divide the
+// conversions among the lanes (coords_float_shared), which costs a call less than the pass and its launch:
+// 32,768 positions x 16 orbitals, 48^3 26.8 -> 24.0 us (Hessian Laplacian 18.4 -> 14.4), 9,000 x 16 12.3 -> 10.2,
+// 12,000 x 128 47.2 -> 45.1, 24,000 x 64 47.5 -> 45.1, 24,000 x 128 bfloat16 61.0 -> 59.1.  The large shape has
+// no such form, and there the pass is the faster one: 30,000 x 128 102 us against 116, 30,000 x 64 58 against
+// 65.  So it is for several tiles of one or two lanes, which would each reduce all three axes: 12,000 x 109
+// bfloat16 37.1 us against 39.7, 40,000 x 40 62.7 against 62.6.
+bool eval_shares_coordinates(const Handle* h, long long n_pos)
+{
+    if (h->storage != QMCSPL_F32 && h->storage != QMCSPL_BF16) return false;
+    if (h->method == QMCSPL_LAGRANGE || h->method == QMCSPL_PPSPLINE || h->separate_grad || is_general(h)) return false;
+    if (h->bloch || h->block_threads == 640 || (h->lanes_log2 < 2 && h->tiles > 1)) return false;
+    const int gpw = 32 >> h->lanes_log2;
+    const long long warps = (n_pos * h->tiles + gpw - 1) / gpw;
+    return warps < (long long)kLargeLaunchRounds * sm_count() * (640 / 32);
+}
 
 int launch_bspline_vgl(const Handle* h, const double* pos, const Prepared& pr, long long n_pos, void* val,
                        void* grad, void* lap, cudaStream_t st)

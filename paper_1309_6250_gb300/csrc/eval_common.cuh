@@ -501,15 +501,14 @@ __device__ __forceinline__ void reduced_coordinates_df(const EvalArgs& p, const 
 // The same reduction for kernels of launches without records, with the double-to-pair conversions
 // divided among the lanes: a conversion is four FP64 instructions, each 64 cycles of a warp's
 // sub-partition, and with every lane converting the position and its row of a^-1 a task spent 24 of
-// them before its first load (a position of 128 orbitals: 1,500 of some 8,000 cycles).  Here lane j < 9
-// converts a^-1's entry j, and lane j < 3 of a group component j of its position; shuffles hand them
-// round.  Same values, same steps, same bits.  4,096 positions x 128 orbitals in input order: 27.8 -> 24.9 us
+// them before its first load (a position of 128 orbitals: 1,500 of some 8,000 cycles).  Here lane j < 3
+// of a group converts component j of its position, the host a^-1; shuffles hand them round.  Same values, same steps, same bits.  4,096 positions x 128 orbitals in input order: 27.8 -> 24.9 us
 // with the Laplacian table, 18.5 -> 14.0 us without; 8,191 x 40: 30.9 -> 22.2 us.
 __device__ __forceinline__ void coords_float_shared(const EvalArgs& p, long long ip, int L, int sub, int gbase, int& ix,
                                                     int& iy, int& iz, float& tx, float& ty, float& tz, bool& ok)
 {
     const int lane = threadIdx.x & 31;
-    const dfloat a = df_from_double(p.ainv[lane < 9 ? lane : 8]);
+    const dfloat a = {p.ainvh[lane < 9 ? lane : 8], p.ainvl[lane < 9 ? lane : 8]};
     const double* pos = p.pos + 3 * ip;
     if (L >= 4) {
         const int ax = sub < 3 ? sub : 2;

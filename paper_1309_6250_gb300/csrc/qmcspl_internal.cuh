@@ -65,8 +65,8 @@ struct EvalArgs {
     double mg[9];             // grad_cart[a] = sum_i mg[3a+i] grad_t[i]
     double ml[6];             // lap = ml0 Hxx + ml1 Hyy + ml2 Hzz + ml3 Hxy + ml4 Hxz + ml5 Hyz
     float mgf[9], mlf[6];     // the same rounded to float (float kernels)
-    float mgh[9], mgl[9];     // double-float split of mg: mg = mgh + mgl
-    float mlh[6], mll[6];     // double-float split of ml
+    float mgl[9], mll[6];     // what the rounding left: mg = mgf + mgl, ml = mlf + mll in double-float
+    float ainvh[9], ainvl[9]; // ainv = ainvh + ainvl in double-float
     float zero;               // 0, where the compiler must not know it (df_mad2)
     const double* pos;
     const void* rec;          // per-position coordinate records (null: compute from pos), see order.cu
@@ -246,6 +246,10 @@ int upload_grid_points(Handle* h, cudaStream_t stream);
 
 // fill the common part of EvalArgs from a handle
 void fill_eval_args(const Handle* h, EvalArgs* a);
+
+// True when the evaluation of n_pos positions in input order takes a kernel that reduces their
+// coordinates as fast as a pass of its own would (eval_bspline.cu).
+bool eval_shares_coordinates(const Handle* h, long long n_pos);
 
 // number of SMs of the current device (cached)
 int sm_count();
