@@ -544,11 +544,12 @@ __global__ void __launch_bounds__(DposShape<T>::threads, 1) bspline_dpos_kernel(
 // Threads per block, positions staged at a time and blocks per SM.  Float: two blocks of 256 threads on
 // an SM, so that one block's staging and barriers overlap the other's columns (the pass at 262,144
 // positions x 128 orbitals: 1.14 ms; one block of 512 threads and batches of 64: 1.33 ms); double
-// staging is too large for two.
-template <typename A> struct GatherShape {
+// staging is too large for two.  WIDE: one block of 512 threads, for double and where it leaves fewer SMs
+// idle (coarse grids: few bins of many positions).
+template <typename A, bool WIDE> struct GatherShape {
     static constexpr int threads = 256, batch = 40, per_sm = 2;
 };
-template <> struct GatherShape<double> {
+template <typename A> struct GatherShape<A, true> {
     static constexpr int threads = 512, batch = 64, per_sm = 1;
 };
 constexpr int kGatherSide = 7;                        // stencil points per axis of a 4-cell bin edge
@@ -617,9 +618,9 @@ struct GatherArgs {
 };
 
 // staged data of one batch (dynamic shared memory)
-template <typename A>
+template <typename A, bool WIDE>
 struct GatherStage {
-    static constexpr int kGatherBatch = GatherShape<A>::batch;
+    static constexpr int kGatherBatch = GatherShape<A, WIDE>::batch;
     static constexpr int EA = 16 / sizeof(A);        // upstream values per 16-byte chunk
     A w[kGatherBatch][3][12];                        // per axis b[4], b'[4], b''[4]
     int cell[kGatherBatch];                          // local cell cx | cy << 8 | cz << 16, -1: none
@@ -627,15 +628,15 @@ struct GatherStage {
     int next;                                        // next column of the batch to take
 };
 
-template <typename A, bool LAPTAB>
-__global__ void __launch_bounds__(GatherShape<A>::threads, GatherShape<A>::per_sm)
+template <typename A, bool LAPTAB, bool WIDE>
+__global__ void __launch_bounds__(GatherShape<A, WIDE>::threads, GatherShape<A, WIDE>::per_sm)
     bspline_bwd_gather_kernel(const BwdArgs b, const GatherArgs g)
 {
-    constexpr int EA = GatherStage<A>::EA;
-    constexpr int WARPS = GatherShape<A>::threads / 32;
-    constexpr int kGatherBatch = GatherShape<A>::batch;
+    constexpr int EA = GatherStage<A, WIDE>::EA;
+    constexpr int WARPS = GatherShape<A, WIDE>::threads / 32;
+    constexpr int kGatherBatch = GatherShape<A, WIDE>::batch;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    GatherStage<A>& S = *reinterpret_cast<GatherStage<A>*>(smem_raw);
+    GatherStage<A, WIDE>& S = *reinterpret_cast<GatherStage<A, WIDE>*>(smem_raw);
     const EvalArgs& p = b.e;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n_orb = p.n_orb;
@@ -823,18 +824,31 @@ int launch_dpos(const BwdArgs& a, cudaStream_t st)
     return cuda_error(cudaGetLastError(), "bspline_dpos_kernel launch");
 }
 
+template <typename A, bool LAPTAB, bool WIDE>
+int launch_gather_shape(const BwdArgs& a, const GatherArgs& g, cudaStream_t st)
+{
+    constexpr size_t smem = sizeof(GatherStage<A, WIDE>);
+    auto k = bspline_bwd_gather_kernel<A, LAPTAB, WIDE>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_error(e, "gathered adjoint shared memory");
+    const int items = g.n_bins * g.n_slices;
+    const int cap = sm_count() * GatherShape<A, WIDE>::per_sm;
+    const int blocks = items < cap ? items : cap;
+    k<<<blocks > 0 ? blocks : 1, GatherShape<A, WIDE>::threads, smem, st>>>(a, g);
+    return cuda_error(cudaGetLastError(), "bspline_bwd_gather_kernel launch");
+}
+
+// Float: the shape with the shorter schedule, a round of two small blocks per SM taking 1.72 times a
+// round of one wide block (GatherShape's figures for 2 x 1.14 / 1.33 ms).
 template <typename A, bool LAPTAB>
 int launch_gather(const BwdArgs& a, const GatherArgs& g, cudaStream_t st)
 {
-    constexpr size_t smem = sizeof(GatherStage<A>);
-    cudaError_t e = cudaFuncSetAttribute(bspline_bwd_gather_kernel<A, LAPTAB>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_error(e, "gathered adjoint shared memory");
-    const int items = g.n_bins * g.n_slices;
-    const int cap = sm_count() * GatherShape<A>::per_sm;
-    const int blocks = items < cap ? items : cap;
-    bspline_bwd_gather_kernel<A, LAPTAB><<<blocks > 0 ? blocks : 1, GatherShape<A>::threads, smem, st>>>(a, g);
-    return cuda_error(cudaGetLastError(), "bspline_bwd_gather_kernel launch");
+    if constexpr (sizeof(A) == 4) {
+        const long long items = (long long)g.n_bins * g.n_slices, sms = sm_count();
+        const long long wide = (items + sms - 1) / sms, small = (items + 2 * sms - 1) / (2 * sms);
+        if (100 * wide > 172 * small) return launch_gather_shape<A, LAPTAB, false>(a, g, st);
+    }
+    return launch_gather_shape<A, LAPTAB, true>(a, g, st);
 }
 
 template <typename T, bool LAPTAB>
