@@ -839,14 +839,17 @@ int launch_gather_shape(const BwdArgs& a, const GatherArgs& g, cudaStream_t st)
 }
 
 // Float: the shape with the shorter schedule, a round of two small blocks per SM taking 1.72 times a
-// round of one wide block (GatherShape's figures for 2 x 1.14 / 1.33 ms).
+// round of one wide block (GatherShape's figures, 2 x 1.14 / 1.33 ms).  Bins of more than about 35
+// positions, which the small batch does not hold at once, take wide blocks: both adjoints of 48^3 x 64
+// orbitals at 38 positions per bin 471 us against 480, at 46 539 against 560, at 130 1,357 against 1,378;
+// at 32 410 us in small blocks against 420.
 template <typename A, bool LAPTAB>
 int launch_gather(const BwdArgs& a, const GatherArgs& g, cudaStream_t st)
 {
     if constexpr (sizeof(A) == 4) {
         const long long items = (long long)g.n_bins * g.n_slices, sms = sm_count();
         const long long wide = (items + sms - 1) / sms, small = (items + 2 * sms - 1) / (2 * sms);
-        if (100 * wide > 172 * small) return launch_gather_shape<A, LAPTAB, false>(a, g, st);
+        if (a.e.n_pos <= 35LL * g.n_bins && 100 * wide > 172 * small) return launch_gather_shape<A, LAPTAB, false>(a, g, st);
     }
     return launch_gather_shape<A, LAPTAB, true>(a, g, st);
 }
