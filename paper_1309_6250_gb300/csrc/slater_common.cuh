@@ -77,35 +77,22 @@ __device__ __forceinline__ void eliminate2(f32x2& H, f32x2& L, f32x2 fh, f32x2 f
     quick_norm2(H, L);
 }
 
-// (H, L) += x y for double-float x = xh + xl and y = yh + yl (yl only where WIDE): df_fma2's steps
-template <bool WIDE>
-__device__ __forceinline__ void dot2(f32x2& H, f32x2& L, f32x2 xh, f32x2 nxh, f32x2 xl, f32x2 yh, f32x2 yl)
+// Sixteen sums over the warp at once: lane l gets the total of s[l >> 1], added up in the order of a
+// butterfly over lane distances 16, 8, 4, 2, 1.  Each exchange halves the sums a lane still carries, so
+// the sixteen cost 16 FP64 additions instead of 80.
+__device__ __forceinline__ double warp_sum16(double (&s)[16])
 {
-    const f32x2 nP = mul2(nxh, yh);
-    f32x2 E = ffma2(xh, yh, nP);
-    if (WIDE) E = ffma2(xh, yl, E);
-    E = ffma2(xl, yh, E);
-    const f32x2 S = sub2(H, nP);
-    const f32x2 B = sub2(S, H);
-    const f32x2 T1 = sub2(H, sub2(S, B));
-    const f32x2 T2 = add2(nP, B);
-    L = add2(L, add2(sub2(T1, T2), E));
-    H = S;
-}
-
-// sum over the warp of double-float pairs; every lane gets the total
-__device__ __forceinline__ void warp_sum2(f32x2& H, f32x2& L)
-{
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const f32x2 h = __shfl_xor_sync(kFullMask, H, off), l = __shfl_xor_sync(kFullMask, L, off);
-        const f32x2 S = add2(H, h);
-        const f32x2 BB = sub2(S, H);
-        const f32x2 T = add2(sub2(H, sub2(S, BB)), sub2(h, BB));
-        L = add2(T, add2(L, l));
-        H = S;
-        quick_norm2(H, L);
+    for (int h = 8; h > 0; h >>= 1) {
+        const bool up = (lane & (2 * h)) != 0;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const double keep = up ? s[q + h] : s[q], give = up ? s[q] : s[q + h];
+            s[q] = keep + __shfl_xor_sync(kFullMask, give, 2 * h);
+        }
     }
+    return s[0] + __shfl_xor_sync(kFullMask, s[0], 1);
 }
 
 __device__ __forceinline__ void split(float v, float& h, float& l)

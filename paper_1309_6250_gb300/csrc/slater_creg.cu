@@ -6,11 +6,12 @@
 // What bounds it: a complex update is four error-free multiply-adds and two renormalisations, 54
 // packed FP32 operations per two entries: 64 x 64 blocks need 2,048 x 54 / 64 = 1,728 SM clocks per
 // elimination step.  slater_cdf_kernel, which it replaces here, moves 32 bytes of shared memory per
-// entry and step, meets at four barriers, and makes its final sums on the FP64 pipe (two operations
-// per SM clock: 27 % of its time).  Here float orbitals' sums are double-float; sums of double
-// orbitals stay FP64, which holds all of their bits.  Measured, complex float orbitals: 4,096 walkers x
-// (64 + 64) 10.19 -> 5.57 ms, 4,096 x (32 + 32) 3.49 -> 0.92 ms, 4,096 x (12 + 11) 1.37 -> 0.42 ms,
-// 1,024 x (96 + 96) 12.1 -> 4.52 ms; error against 64 bits unchanged in every case.
+// entry and step and meets at four barriers.  The final sums are FP64 here as there (two operations per
+// SM clock): in double-float they had 1.03 to 1.10 times
+// the drift's rms error, and neither a double's last bits nor its range.  Measured, 4,096 walkers x
+// (64 + 64), complex float orbitals 10.18 -> 5.24 ms (5.56 with double-float sums), complex double 9.57 -> 5.39;
+// 4,096 x (32 + 32) 3.49 -> 0.95 ms (0.92), 4,096 x (12 + 11) 1.35 -> 0.41 (0.40), 1,024 x (96 + 96)
+// 12.1 -> 5.39 (4.52).
 //
 // A lane keeps RL rows of CP column pairs, each as four packed pairs (re and im, high and low): 64
 // registers, 72 for 65 to 96 electrons.  97 to 112 electrons would need 98 of 128 and stay with
@@ -294,86 +295,41 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32 * CregShape<G>::N
         odd = __reduce_xor_sync(kFullMask, odd);
         if (lane == 0 && odd) atomicXor(&parity, 1);
         __syncthreads();
-        // T = -1/2 sum_ij X_ji lap phi_j(r_i) and the drift
+        // T = -1/2 sum_ij X_ji lap phi_j(r_i) and the drift, in FP64 (inverse entries h + l): two electrons
+        // per warp at a time, lanes 16 e + 4 c + 2 r and the next getting sum c (r = 0 re, 1 im) of electron e
         const bool want_g = a.drift != nullptr, want_l = a.kinetic != nullptr;
         if (want_g || want_l) {
             const T* gp = static_cast<const T*>(a.grad);
             const T* lp = static_cast<const T*>(a.lap);
-            auto source = [&](int c, int i, int j) __attribute__((always_inline)) {   // quantity c of electron i
-                return c < 3 ? gp + 2 * (((base + i) * 3 + c) * O + j) : lp + 2 * ((base + i) * O + j);
-            };
-            if constexpr (sizeof(T) == 8) {
-                for (int i = wid; i < n; i += NW)
-                    for (int c = want_g ? 0 : 3; c < (want_l ? 4 : 3); ++c) {
-                        double sr = 0.0, si = 0.0;
-                        for (int j = lane; j < n; j += 32) {
-                            const float4 x = xct[i * ld + j];
-                            const double xr = (double)x.x + (double)x.y, xi = (double)x.z + (double)x.w;
-                            const double* s = source(c, i, j);
-                            const double zr = __ldg(s), zi = __ldg(s + 1);
-                            sr += xr * zr - xi * zi;
-                            si += xr * zi + xi * zr;
-                        }
-                        for (int off = 16; off > 0; off >>= 1) {
-                            sr += __shfl_xor_sync(kFullMask, sr, off);
-                            si += __shfl_xor_sync(kFullMask, si, off);
-                        }
-                        if (lane == 0) {
-                            if (c < 3) {
-                                a.drift[2 * ((base + i) * 3 + c)] = sr;
-                                a.drift[2 * ((base + i) * 3 + c) + 1] = si;
-                            } else {
-                                kin_re += sr;
-                                kin_im += si;
-                            }
-                        }
-                    }
-            } else {
-                // the eight sums of an electron as packed pairs (re, im), four electrons per warp at a
-                // time; lane 8 e + 2 c + (0 re, 1 im) keeps a sum, so that the conversions to double run
-                // once for all of them
-                for (int i0 = 4 * wid; i0 < n; i0 += 4 * NW) {
-                    float kh = 0.f, kl = 0.f;
-                    for (int e = 0; e < 4 && i0 + e < n; ++e) {
-                        const int i = i0 + e;
-                        f32x2 Ah[4] = {0ull, 0ull, 0ull, 0ull}, Al[4] = {0ull, 0ull, 0ull, 0ull};
+            for (int i0 = 2 * wid; i0 < n; i0 += 2 * NW) {
+                double s[16];
 #pragma unroll
-                        for (int t = 0; t < RL; ++t) {
-                            const int j = lane + 32 * t;
-                            if (j >= n) continue;
-                            const float4 x = xct[i * ld + j];
-                            const f32x2 xrh = pack2(x.x, x.x), nxrh = pack2(-x.x, -x.x), xrl = pack2(x.y, x.y);
-                            const f32x2 xih = pack2(x.z, x.z), nxih = pack2(-x.z, -x.z), xil = pack2(x.w, x.w);
+                for (int e = 0; e < 2; ++e) {
+                    const int i = i0 + e;
 #pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                if (c < 3 ? !want_g : !want_l) continue;
-                                const T* s = source(c, i, j);
-                                const float zr = __ldg(s), zi = __ldg(s + 1);
-                                dot2<false>(Ah[c], Al[c], xrh, nxrh, xrl, pack2(zr, zi), 0ull);
-                                dot2<false>(Ah[c], Al[c], xih, nxih, xil, pack2(-zi, zr), 0ull);
-                            }
-                        }
+                    for (int c = 0; c < 8; ++c) s[8 * e + c] = 0.0;
+#pragma unroll
+                    for (int t = 0; t < RL; ++t) {
+                        const int j = lane + 32 * t;
+                        if (i >= n || j >= n) continue;
+                        const float4 x = xct[i * ld + j];
+                        const double xr = (double)x.x + (double)x.y, xi = (double)x.z + (double)x.w;
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
-                            warp_sum2(Ah[c], Al[c]);
-                            float h0, h1, l0, l1;
-                            unpack2(Ah[c], h0, h1);
-                            unpack2(Al[c], l0, l1);
-                            if ((lane >> 1) == 4 * e + c) {
-                                kh = (lane & 1) ? h1 : h0;
-                                kl = (lane & 1) ? l1 : l0;
-                            }
+                            if (c < 3 ? !want_g : !want_l) continue;
+                            const T* z = c < 3 ? gp + 2 * (((base + i) * 3 + c) * O + j) : lp + 2 * ((base + i) * O + j);
+                            const double zr = __ldg(z), zi = __ldg(z + 1);
+                            double &sr = s[8 * e + 2 * c], &si = s[8 * e + 2 * c + 1];
+                            sr = fma(xr, zr, fma(-xi, zi, sr));
+                            si = fma(xr, zi, fma(xi, zr, si));
                         }
                     }
-                    const double s = (double)kh + (double)kl;
-                    const int i = i0 + (lane >> 3), c = (lane >> 1) & 3;
-                    if (c == 3) {
-                        if (lane & 1) kin_im += s;
-                        else kin_re += s;
-                    } else if (want_g && i < n) {
-                        a.drift[2 * ((base + i) * 3 + c) + (lane & 1)] = s;
-                    }
                 }
+                const double sum = warp_sum16(s);
+                const int i = i0 + (lane >> 4), c = (lane >> 2) & 3, r = (lane >> 1) & 1;
+                if (lane & 1) continue;
+                if (c == 3) (r ? kin_im : kin_re) += sum;
+                else if (want_g && i < n) a.drift[2 * ((base + i) * 3 + c) + r] = sum;
             }
         }
     }

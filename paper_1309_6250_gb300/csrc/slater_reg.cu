@@ -6,9 +6,12 @@
 // 128 x 128 blocks need 16,384 x 15 / 128 = 1,920 SM clocks per elimination step.  The kernel it
 // replaces kept the matrix in shared memory, where each update also read and wrote 16 bytes, and met
 // at four barriers per step: 14.29 ms for 2,048 walkers x (128 + 128) electrons.  Here the matrix
-// never leaves the registers and the warps meet at no barrier: 5.92 ms (3,190 clocks per step plus
-// 380 for the load and the final sums; FP32 pipe 68 % busy).  64 + 64 electrons: 2.90 -> 0.87 ms,
-// 96 + 96: 6.13 -> 2.48 ms (2,048 walkers); 8 + 8: 0.62 -> 0.13 ms, 32 + 32: 2.25 -> 0.40 ms (4,096).
+// never leaves the registers and the warps meet at no barrier: 6.79 ms.  Of that about 1 ms is the final
+// sums, which stay FP64 (two operations per SM clock): as double-float sums on the FP32 pipe they left
+// 5.87 ms, but the drift's rms error against 64 bits was 1.03 (128 electrons) to 1.18 times (12) as large,
+// a double's last bits were lost and an infinite gradient gave NaN.  64 + 64 electrons: 2.90 -> 0.88 ms,
+// 96 + 96: 6.08 -> 2.50 ms (2,048 walkers); 8 + 8: 0.62 -> 0.14 ms, 32 + 32: 2.24 -> 0.43 ms (4,096);
+// double orbitals, 128 + 128: 13.73 -> 6.63 ms.
 // Also measured, 128 + 128: 32 x 32 tiles per warp, the pivot row and column through shared memory
 // and two barriers per step 7.4 ms (each step's search and scaling lay between the updates, and the
 // few lanes that do them compete with the other warps' updates); columns owned by warps in blocks,
@@ -65,7 +68,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32 * RegShape<G>::NW
     constexpr int N = 32 * RL, NT = 32 * NW, CW = 2 * CP;
     static_assert(CW * NW == N && CW <= 32, "the warps cover the columns, a lane scales one of them");
     constexpr int ld = N + 1;                       // row stride of the inverse in shared memory
-    constexpr bool kWide = sizeof(T) == 8;
     // during the elimination column k's multipliers (h, l), xt[k * N + row]; then the inverse by
     // electron, xt[i * ld + j]
     extern __shared__ float2 xt[];
@@ -297,51 +299,45 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32 * RegShape<G>::NW
         odd = __reduce_xor_sync(kFullMask, odd);
         if (lane == 0 && odd) atomicXor(&parity, 1);
         __syncthreads();
-        // T = -1/2 sum_ij X_ji lap phi_j(r_i) and the drift: eight electrons per warp at a time, the
-        // four sums of an electron as packed pairs; lane 4 e + c keeps sum c of electron e, so that
-        // the conversions to double run once for all of them
+        // T = -1/2 sum_ij X_ji lap phi_j(r_i) and the drift, in FP64 (inverse entries h + l): four electrons
+        // per warp at a time, lanes 8 e + 2 c and the next getting sum c of electron e
         const bool want_g = a.drift != nullptr, want_l = a.kinetic != nullptr;
         if (want_g || want_l) {
             const T* gp = static_cast<const T*>(a.grad);
             const T* lp = static_cast<const T*>(a.lap);
-            for (int i0 = 8 * wid; i0 < n; i0 += 8 * NW) {
-                float kh = 0.f, kl = 0.f;
-                for (int e = 0; e < 8 && i0 + e < n; ++e) {
+            for (int i0 = 4 * wid; i0 < n; i0 += 4 * NW) {
+                double s[16];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
                     const int i = i0 + e;
-                    f32x2 Ah = 0ull, Al = 0ull, Bh = 0ull, Bl = 0ull;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) s[4 * e + c] = 0.0;
+                    if (i >= n) continue;
+                    float2 z[RL];
+                    T g[RL][4];                     // all of an electron's loads first
 #pragma unroll
                     for (int t = 0; t < RL; ++t) {
                         const int jj = lane + 32 * t;
-                        if (jj >= n) continue;
-                        const float2 x = xt[(size_t)i * ld + jj];
-                        const f32x2 xh = pack2(x.x, x.x), nxh = pack2(-x.x, -x.x), xl = pack2(x.y, x.y);
-                        float g[3][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}}, q[2] = {0.f, 0.f};
-                        if (want_g)
+                        const bool on = jj < n;
+                        z[t] = on ? xt[(size_t)i * ld + jj] : make_float2(0.0f, 0.0f);
 #pragma unroll
-                            for (int c = 0; c < 3; ++c)
-                                split(__ldg(gp + ((base + i) * 3 + c) * O + jj), g[c][0], g[c][1]);
-                        if (want_l) split(__ldg(lp + (base + i) * O + jj), q[0], q[1]);
-                        dot2<kWide>(Ah, Al, xh, nxh, xl, pack2(g[0][0], g[1][0]), pack2(g[0][1], g[1][1]));
-                        dot2<kWide>(Bh, Bl, xh, nxh, xl, pack2(g[2][0], q[0]), pack2(g[2][1], q[1]));
+                        for (int c = 0; c < 3; ++c) g[t][c] = on && want_g ? __ldg(gp + ((base + i) * 3 + c) * O + jj) : T(0);
+                        g[t][3] = on && want_l ? __ldg(lp + (base + i) * O + jj) : T(0);
                     }
-                    warp_sum2(Ah, Al);
-                    warp_sum2(Bh, Bl);
-                    float h[4], l[4];
-                    unpack2(Ah, h[0], h[1]);
-                    unpack2(Al, l[0], l[1]);
-                    unpack2(Bh, h[2], h[3]);
-                    unpack2(Bl, l[2], l[3]);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        if (lane == 4 * e + c) {
-                            kh = h[c];
-                            kl = l[c];
-                        }
+                    for (int t = 0; t < RL; ++t) {
+                        if (32 * t >= n) continue;
+                        const double x = (double)z[t].x + (double)z[t].y;
+#pragma unroll
+                        for (int c = 0; c < 4; ++c)
+                            if (c < 3 ? want_g : want_l) s[4 * e + c] = fma(x, (double)g[t][c], s[4 * e + c]);
+                    }
                 }
-                const double s = (double)kh + (double)kl;
-                const int i = i0 + (lane >> 2), c = lane & 3;
-                if (c == 3) part_kin += s;
-                else if (want_g && i < n) a.drift[(base + i) * 3 + c] = s;
+                const double sum = warp_sum16(s);
+                const int i = i0 + (lane >> 3), c = (lane >> 1) & 3;
+                if (lane & 1) continue;
+                if (c == 3) part_kin += sum;
+                else if (want_g && i < n) a.drift[(base + i) * 3 + c] = sum;
             }
         }
     }
