@@ -226,8 +226,10 @@ __global__ void __launch_bounds__(kSlaterThreads) slater_kernel(const SlaterArgs
 // (smaller ones: slater_reg.cu, the matrix in registers).  Shared memory holds the matrix as two float arrays
 // Ah, Al of [n][ns] with ns = n rounded up to even, plus 2 (zero padding columns stay zero
 // through the elimination), so that column pairs (j, j+1) are one 8-byte word of each.
+// (One CTA per SM by shared memory, so 102 registers cost nothing; without the 1 the compiler keeps to
+// 64 and spills: 1,024 walkers x (144 + 144) 15.95 ms instead of 15.12.)
 template <typename T, int NT>
-__global__ void __launch_bounds__(NT) slater_df_kernel(const SlaterArgs a)
+__global__ void __launch_bounds__(NT, 1) slater_df_kernel(const SlaterArgs a)
 {
     extern __shared__ float fsm[];
     __shared__ double red[NT / 32];
