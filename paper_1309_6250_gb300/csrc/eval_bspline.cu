@@ -708,10 +708,11 @@ template <typename T, bool LAPTAB, int THREADS>
 int launch_shape(const EvalArgs& a, long long warps, cudaStream_t st)
 {
     auto k = bspline_vgl_kernel<T, LAPTAB, THREADS, false>;
-    if constexpr (kStaged<T>) {
-        if (!a.vec_out) k = bspline_vgl_kernel<T, LAPTAB, THREADS, true>;
+    if constexpr (Traits<T>::E >= 4) {
+        const bool staged = staged_rows<T>(a, warps, LAPTAB ? 10 : 6);
+        if (staged) k = bspline_vgl_kernel<T, LAPTAB, THREADS, true>;
         if constexpr (THREADS == QMCSPL_EVAL_THREADS) {   // (the large shape's launches have records)
-            if (!a.rec) k = a.vec_out ? bspline_vgl_kernel<T, LAPTAB, THREADS, false, true> : bspline_vgl_kernel<T, LAPTAB, THREADS, true, true>;
+            if (!a.rec) k = staged ? bspline_vgl_kernel<T, LAPTAB, THREADS, true, true> : bspline_vgl_kernel<T, LAPTAB, THREADS, false, true>;
         }
     }
     k<<<(unsigned)grid_for(k, THREADS, warps), THREADS, 0, st>>>(a);
@@ -735,9 +736,12 @@ int launch_small(const EvalArgs& a, long long warps, cudaStream_t st)
         }
     }
     auto k = bspline_vgl_small_kernel<T, LAPTAB, false>;
-    if constexpr (kStaged<T>) {
-        if (!a.vec_out) k = a.rec ? bspline_vgl_small_kernel<T, LAPTAB, true> : bspline_vgl_small_kernel<T, LAPTAB, true, true>;
-        else if (!a.rec) k = bspline_vgl_small_kernel<T, LAPTAB, false, true>;
+    if constexpr (Traits<T>::E >= 4) {
+        if (!a.rec) k = bspline_vgl_small_kernel<T, LAPTAB, false, true>;
+    }
+    if constexpr (Traits<T>::E == 8) {
+        if (staged_rows<T>(a, warps, 0))
+            k = a.rec ? bspline_vgl_small_kernel<T, LAPTAB, true> : bspline_vgl_small_kernel<T, LAPTAB, true, true>;
     }
     k<<<(unsigned)warps, 32, 0, st>>>(a);
     return cuda_error(cudaGetLastError(), "bspline_vgl_small_kernel launch");

@@ -758,9 +758,25 @@ struct RaggedStore {
     }
 };
 
-// RAGGED kernels (float and bfloat16 tables) store through it: floats of shared memory per warp.
+// RAGGED kernels store through it: floats of shared memory per warp.
 template <typename T, bool RAGGED> constexpr int kStageFloats = RAGGED ? 32 * Traits<T>::E : 4;
-template <typename T> constexpr bool kStaged = Traits<T>::E >= 4;
+// Which launches of `warps` warp tasks with unaligned rows do.  A lane of a bfloat16 table holds eight floats
+// of a row: scalar stores took 1.05 to 1.7 times as long (9 to 150 orbitals, 9,000 to 120,000 positions, 32^3 to
+// 80^3, every basis), but with fewer than three warp tasks on an SM nothing queues for the stores and the staging
+// only adds its latency (2,000 positions x 21 orbitals, Hessian Laplacian, 9.1 us direct, 10.6 staged; 9,000 x 21
+// 15.1 direct, 13.9 staged).  A lane of a float table holds four: scalar stores hide behind the gather of many
+// chunks, where the staging does not (60,000 x 63, 64^3, Hessian Laplacian, 80.4 us direct, 90.2 staged; 30,000 x
+// 150 with the Laplacian table, 80^3, 179 direct, 203 staged), and behind the few warps of a small launch.
+// Positions of few chunks gain: 120,000 x 37, 48^3, Laplacian table, 168.8 us direct, 154.2 staged; 60,000 x 21,
+// Hessian 1.02 to 1.06 times.  float_chunks, the most for which that was so: 10 with the Laplacian table, 6 with the
+// Hessian Laplacian; float five-table and pp kernels gain nothing (within 2 %, 5 % the other way at 63 orbitals).
+template <typename T> bool staged_rows(const EvalArgs& a, long long warps, int float_chunks)
+{
+    constexpr int E = Traits<T>::E;
+    if (a.vec_out) return false;
+    if (E == 8) return warps >= 3LL * sm_count();
+    return E == 4 && !small_launch(warps) && (a.n_orb + E - 1) / E <= float_chunks;
+}
 
 // Streaming stores of E consecutive outputs (vector when allowed).
 template <typename A, int E>

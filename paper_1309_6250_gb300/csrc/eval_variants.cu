@@ -643,12 +643,17 @@ __global__ void __launch_bounds__(THREADS, THREADS == 32 ? kSmallWarps : 1) pp_v
     }
 }
 
+long long warp_tasks(const EvalArgs& a)
+{
+    const int gpw = 32 >> a.lanes_log2;
+    return (a.n_pos * a.tiles + gpw - 1) / gpw;
+}
+
 // `small`: the same kernel with a block per warp task, for small launches
 template <typename K>
 int launch_one_block_per_sm(K kernel, K small, int threads, const EvalArgs& a, cudaStream_t st, const char* name)
 {
-    const int gpw = 32 >> a.lanes_log2;
-    const long long warps = (a.n_pos * a.tiles + gpw - 1) / gpw;
+    const long long warps = warp_tasks(a);
     if (small_launch(warps)) {
         small<<<(unsigned)warps, 32, 0, st>>>(a);
         return cuda_error(cudaGetLastError(), name);
@@ -676,8 +681,8 @@ int launch_five_rows(const EvalArgs& a, cudaStream_t st)
 template <typename T, int BASIS>
 int launch_five(const EvalArgs& a, cudaStream_t st)
 {
-    if constexpr (kStaged<T>) {
-        if (!a.vec_out) return launch_five_rows<T, BASIS, true>(a, st);
+    if constexpr (Traits<T>::E == 8) {
+        if (staged_rows<T>(a, warp_tasks(a), 0)) return launch_five_rows<T, BASIS, true>(a, st);
     }
     return launch_five_rows<T, BASIS, false>(a, st);
 }
@@ -692,8 +697,8 @@ int launch_pp_rows(const EvalArgs& a, cudaStream_t st)
 template <typename T>
 int launch_pp(const EvalArgs& a, cudaStream_t st)
 {
-    if constexpr (kStaged<T>) {
-        if (!a.vec_out) return launch_pp_rows<T, true>(a, st);
+    if constexpr (Traits<T>::E == 8) {
+        if (staged_rows<T>(a, warp_tasks(a), 0)) return launch_pp_rows<T, true>(a, st);
     }
     return launch_pp_rows<T, false>(a, st);
 }
