@@ -524,7 +524,9 @@ int qmcspl_eval_vgl_noalloc(qmcspl_t h, const double* pos, long long n_pos, void
  * block per walker, in FP64 or in double-float (arith); complex entries are pivoted on the
  * largest modulus, and in double-float each of their parts is a float pair.  An exactly
  * singular block gives sign 0, logdet -inf and NaN kinetic energy and drift for that walker;
- * nearly singular blocks lose accuracy as the condition number grows.
+ * nearly singular blocks lose accuracy as the condition number grows.  In the double-float kernels
+ * for up to 128 electrons per block (96 for complex dtypes) warps wait for one another's pivot
+ * columns; should such a wait run out, every output of its walker is NaN, sign and logdet included.
  */
 #define QMCSPL_SLATER_MAX_BLOCK 160
 #define QMCSPL_SLATER_MAX_COMPLEX_BLOCK 112
@@ -559,6 +561,16 @@ int qmcspl_debug_fail_alloc(long long n);
  * QMCSPL_OK.
  */
 int qmcspl_debug_stall_pipeline(int n);
+
+/*
+ * qmcspl_debug_stall_slater -- test hook: in the next n qmcspl_slater_kinetic calls that run the
+ * double-float kernels with the matrix in registers, the first pivot column of the first walker's
+ * first spin block is never announced, so that the waits for it run out (within about a second)
+ * exactly as they would if a warp had stalled.  The launch then ends on its own; every output of
+ * that walker is NaN, whatever its matrix, and the other walkers' are as ever.  n <= 0 switches the
+ * hook off.  Returns QMCSPL_OK.
+ */
+int qmcspl_debug_stall_slater(int n);
 
 /*
  * qmcspl_profile / qmcspl_profile_read -- CUDA-event timing of the library's own kernels.

@@ -121,6 +121,7 @@ PROTOTYPES = [
     ("qmcspl_slater_kinetic", I, [VP, VP, VP, I, I, LL, I, I, I, VP, VP, VP, VP, VP]),
     ("qmcspl_debug_fail_alloc", I, [LL]),
     ("qmcspl_debug_stall_pipeline", I, [I]),
+    ("qmcspl_debug_stall_slater", I, [I]),
     ("qmcspl_probe_cache", I, [I, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double),
                                ctypes.POINTER(ctypes.c_double), VP]),
     ("qmcspl_probe_fma", I, [I, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double),

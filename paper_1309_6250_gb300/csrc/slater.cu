@@ -25,6 +25,7 @@
 // Complex orbitals (Bloch functions) take a complex elimination, in FP64 (slater_complex_kernel)
 // or in double-float (slater_cdf_kernel).  The double-float kernels here serve the largest spin blocks;
 // smaller ones keep their matrix in registers (slater_reg.cu, slater_creg.cu).
+#include <atomic>
 #include <cmath>
 
 #include "slater_common.cuh"
@@ -982,6 +983,14 @@ int launch_slater(const SlaterArgs& a, int nmax, cudaStream_t st)
 
 using namespace qmcspl;
 
+static std::atomic<int> g_stall_launches{0};
+
+extern "C" int qmcspl_debug_stall_slater(int n)
+{
+    g_stall_launches.store(n > 0 ? n : 0);
+    return QMCSPL_OK;
+}
+
 extern "C" int qmcspl_slater_kinetic(const void* val, const void* grad, const void* lap, int dtype, int arith,
                                      long long n_walkers, int n_elec, int n_up, int n_orb, double* logdet,
                                      double* sign, double* kinetic, double* drift, void* stream)
@@ -1017,6 +1026,13 @@ extern "C" int qmcspl_slater_kinetic(const void* val, const void* grad, const vo
     a.kinetic = kinetic;
     a.drift = drift;
     a.arith = arith;
+    a.stall = 0;
+    if (arith == QMCSPL_SLATER_DF64 && nmax <= (cplx ? kSlaterCregMaxBlock : kSlaterRegMaxBlock))
+        for (int v = g_stall_launches.load(); v > 0;)
+            if (g_stall_launches.compare_exchange_weak(v, v - 1)) {
+                a.stall = 1;
+                break;
+            }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     switch (dtype) {
     case 0: return launch_slater<double>(a, nmax, st);

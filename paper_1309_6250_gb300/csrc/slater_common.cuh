@@ -21,6 +21,7 @@ struct SlaterArgs {
     double* kinetic;
     double* drift;
     int arith;                // 0: FP64, 1: double-float
+    int stall;                // test hook: column 0 of the first walker's first block is never announced
 };
 
 // The double-float consumer for spin blocks of at most kSlaterRegMaxBlock electrons: real
@@ -107,10 +108,11 @@ __device__ __forceinline__ void split(double v, float& h, float& l)
     l = d.l;
 }
 
-// ---- mbarriers (one arrival each, never reused) ----
-__device__ __forceinline__ void mbar_init(uint64_t* bar)
+// ---- mbarriers (one arrival each, never reused; the test hook's barrier expects a second one) ----
+__device__ __forceinline__ void mbar_init(uint64_t* bar, int arrivals)
 {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(bar)) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(bar)), "r"(arrivals)
+                 : "memory");
 }
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
 {

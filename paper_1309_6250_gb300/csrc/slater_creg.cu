@@ -92,7 +92,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32 * CregShape<G>::N
     const long long base = w * a.n_elec + e0;       // first position of the block
     const long long O = a.n_orb;
     if (tid == 0) parity = 0;
-    for (int k = tid; k < N; k += NT) mbar_init(ready + k);
+    for (int k = tid; k < N; k += NT) mbar_init(ready + k, a.stall && k == 0 && w == 0 && spin == 0 ? 2 : 1);
 
     CplxEntry2 X[RL][CP];                           // [row lane + 32 i][column pair]
     {
@@ -183,10 +183,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32 * CregShape<G>::N
     int fail = 0;                                   // 1: singular, 2: a wait ran out
 #pragma unroll 1
     for (int k = 0; k < n && wid < n; ++k) {
-        if (!mbar_wait(ready + k)) fail = 2;
+        const bool there = mbar_wait(ready + k);
         __syncwarp();                               // (step k - 1's row is read by all lanes)
         const int p = piv[k];
-        if (p < 0) fail = 1;                        // exactly singular
+        if (!there) fail = 2;                       // (nothing is known about piv[k])
+        else if (p < 0) fail = 1;                   // exactly singular
         if (__any_sync(kFullMask, fail)) break;
         const bool mine_row = lane == (p & 31);
 #pragma unroll

@@ -91,7 +91,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32 * RegShape<G>::NW
     const long long base = w * a.n_elec + e0;       // first position of the block
     const long long O = a.n_orb;
     if (tid == 0) parity = 0;
-    for (int k = tid; k < N; k += NT) mbar_init(ready + k);
+    for (int k = tid; k < N; k += NT) mbar_init(ready + k, a.stall && k == 0 && w == 0 && spin == 0 ? 2 : 1);
 
     f32x2 H[RL][CP], L[RL][CP];                     // [row lane + 32 i][column pair]
     {
@@ -162,11 +162,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32 * RegShape<G>::NW
     int fail = 0;                                   // 1: singular, 2: a wait ran out
 #pragma unroll 1
     for (int k = 0; k < n && wid < n; ++k) {
-        if (!mbar_wait(ready + k)) fail = 2;
+        const bool there = mbar_wait(ready + k);
         __syncwarp();                               // (step k - 1's row is read by all lanes)
         const float4 ct = ctrl[k];
         const int p = __float_as_int(ct.x);
-        if (p < 0) fail = 1;                        // exactly singular
+        if (!there) fail = 2;                       // (nothing is known about ctrl[k])
+        else if (p < 0) fail = 1;                   // exactly singular
         if (__any_sync(kFullMask, fail)) break;
         const bool mine_row = lane == (p & 31);
 #pragma unroll
