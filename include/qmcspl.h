@@ -526,7 +526,8 @@ int qmcspl_eval_vgl_noalloc(qmcspl_t h, const double* pos, long long n_pos, void
  * singular block gives sign 0, logdet -inf and NaN kinetic energy and drift for that walker;
  * nearly singular blocks lose accuracy as the condition number grows.  In the double-float kernels
  * for up to 128 electrons per block (96 for complex dtypes) warps wait for one another's pivot
- * columns; should such a wait run out, every output of its walker is NaN, sign and logdet included.
+ * columns; should such a wait run out, every output of its walker is NaN, sign and logdet included,
+ * and qmcspl_slater_sync reports it.
  */
 #define QMCSPL_SLATER_MAX_BLOCK 160
 #define QMCSPL_SLATER_MAX_COMPLEX_BLOCK 112
@@ -540,6 +541,16 @@ enum qmcspl_slater_arith {
 int qmcspl_slater_kinetic(const void* val, const void* grad, const void* lap, int dtype, int arith,
                           long long n_walkers, int n_elec, int n_up, int n_orb, double* logdet, double* sign,
                           double* kinetic, double* drift, void* stream);
+
+/*
+ * qmcspl_slater_sync -- wait for the consumer calls on `stream` (a cudaStream_t of the current
+ * device) and report.
+ *
+ * Returns QMCSPL_ERR_TIMEOUT if, since the last report, a wait inside a consumer launch that is
+ * done by then on this device (any stream) ran out, so that some walker's outputs are NaN for that
+ * reason; QMCSPL_OK otherwise.  Reading the outputs needs no such call.
+ */
+int qmcspl_slater_sync(void* stream);
 
 /*
  * qmcspl_debug_fail_alloc -- test hook: make one device allocation of the library fail.

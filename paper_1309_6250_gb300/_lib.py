@@ -119,6 +119,7 @@ PROTOTYPES = [
     ("qmcspl_save", I, [VP, ctypes.c_char_p]),
     ("qmcspl_load", I, [ctypes.POINTER(VP), ctypes.c_char_p, VP]),
     ("qmcspl_slater_kinetic", I, [VP, VP, VP, I, I, LL, I, I, I, VP, VP, VP, VP, VP]),
+    ("qmcspl_slater_sync", I, [VP]),
     ("qmcspl_debug_fail_alloc", I, [LL]),
     ("qmcspl_debug_stall_pipeline", I, [I]),
     ("qmcspl_debug_stall_slater", I, [I]),

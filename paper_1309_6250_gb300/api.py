@@ -351,3 +351,10 @@ def slater_kinetic(val: torch.Tensor, grad: Optional[torch.Tensor], lap: Optiona
                                              n_orb, _ptr(logdet), _ptr(sign), _ptr(kin), _ptr(drift),
                                              _stream_handle(stream)))
     return logdet, sign, kin, drift
+
+
+def slater_sync(stream=None, device=None) -> None:
+    """Wait for the consumer calls on `stream` (default: the current one of `device`); raises QmcsplError
+    (ERR_TIMEOUT) if a wait inside one of the device's consumer launches ran out since the last report."""
+    with torch.cuda.device(device if device is not None else torch.cuda.current_device()):
+        _lib.check(_lib.load().qmcspl_slater_sync(_stream_handle(stream)))

@@ -1041,3 +1041,23 @@ extern "C" int qmcspl_slater_kinetic(const void* val, const void* grad, const vo
     default: return launch_slater_complex<float>(a, nmax, st);
     }
 }
+
+extern "C" int qmcspl_slater_sync(void* stream)
+{
+    clear_error();
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    int flags[2] = {0, 0};
+    void* word[2];
+    cudaError_t e = slater_reg_timeout_word(&word[0]);
+    if (e == cudaSuccess) e = slater_creg_timeout_word(&word[1]);
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i)
+        e = cudaMemcpyAsync(&flags[i], word[i], sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i)
+        if (flags[i]) e = cudaMemsetAsync(word[i], 0, sizeof(int), st);
+    if (e == cudaSuccess && (flags[0] || flags[1])) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_error(e, "qmcspl_slater_sync");
+    if (flags[0] || flags[1])
+        return set_error(QMCSPL_ERR_TIMEOUT, "a wait of the Slater consumer gave up: its walker's outputs are NaN");
+    return QMCSPL_OK;
+}

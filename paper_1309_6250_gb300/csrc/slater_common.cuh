@@ -31,6 +31,9 @@ int launch_slater_reg_f32(const SlaterArgs& a, int nmax, cudaStream_t st);
 // The same for complex orbitals and at most kSlaterCregMaxBlock electrons (slater_creg.cu).
 int launch_slater_creg_f64(const SlaterArgs& a, int nmax, cudaStream_t st);
 int launch_slater_creg_f32(const SlaterArgs& a, int nmax, cudaStream_t st);
+// Address of each file's device word, set by a walker whose waits ran out.
+cudaError_t slater_reg_timeout_word(void** p);
+cudaError_t slater_creg_timeout_word(void** p);
 
 namespace {
 

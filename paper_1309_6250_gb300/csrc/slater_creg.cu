@@ -25,6 +25,8 @@ namespace {
 
 namespace cg = cooperative_groups;
 
+__device__ int timed_out;   // read and cleared by qmcspl_slater_sync
+
 // G: spin blocks of at most 32 G electrons; see RegShape in slater_reg.cu
 template <int G> struct CregShape;
 template <> struct CregShape<1> { static constexpr int RL = 1, CP = 8, NW = 2, per_sm = 8; };
@@ -362,6 +364,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32 * CregShape<G>::N
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
     const double inf = __longlong_as_double(0x7ff0000000000000LL);
     if (spin == 0 && tid == 0) {
+        if (lost) timed_out = 1;
         if (a.logdet) a.logdet[w] = lost ? nan : singular ? -inf : mine.logdet + other.logdet;
         if (a.sign) {
             double sn, cs;
@@ -406,6 +409,8 @@ int launch_typed(const SlaterArgs& a, int nmax, cudaStream_t st)
 }
 
 }  // namespace
+
+cudaError_t slater_creg_timeout_word(void** p) { return cudaGetSymbolAddress(p, timed_out); }
 
 int launch_slater_creg_f64(const SlaterArgs& a, int nmax, cudaStream_t st) { return launch_typed<double>(a, nmax, st); }
 int launch_slater_creg_f32(const SlaterArgs& a, int nmax, cudaStream_t st) { return launch_typed<float>(a, nmax, st); }

@@ -45,6 +45,8 @@ namespace {
 
 namespace cg = cooperative_groups;
 
+__device__ int timed_out;   // read and cleared by qmcspl_slater_sync
+
 // RL rows per lane, CP column pairs per lane, NW warps; `per_sm` CTAs of at most 128 registers per
 // thread fit on an SM.  G: spin blocks of at most 32 G electrons.
 template <int G> struct RegShape;
@@ -363,6 +365,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32 * RegShape<G>::NW
     const bool singular = sing || other.singular;
     const bool lost = stuck || other.stuck;
     if (spin == 0 && tid == 0) {
+        if (lost) timed_out = 1;
         const double nan = __longlong_as_double(0x7ff8000000000000LL);
         const double inf = __longlong_as_double(0x7ff0000000000000LL);
         if (a.logdet) a.logdet[w] = lost ? nan : singular ? -inf : logdet + other.logdet;
@@ -407,6 +410,8 @@ int launch_typed(const SlaterArgs& a, int nmax, cudaStream_t st)
 }
 
 }  // namespace
+
+cudaError_t slater_reg_timeout_word(void** p) { return cudaGetSymbolAddress(p, timed_out); }
 
 int launch_slater_reg_f64(const SlaterArgs& a, int nmax, cudaStream_t st) { return launch_typed<double>(a, nmax, st); }
 int launch_slater_reg_f32(const SlaterArgs& a, int nmax, cudaStream_t st) { return launch_typed<float>(a, nmax, st); }

@@ -36,3 +36,31 @@ def test_stalled_walker_is_nan(cplx, n_up, n_dn, singular):
         assert torch.isnan(torch.view_as_real(a[0]) if a.is_complex() else a[0]).all()
         assert torch.equal(a[1:], b[1:]) and torch.equal(c[1:], b[1:])
         np.testing.assert_array_equal(c[0].cpu().numpy(), b[0].cpu().numpy())
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+def test_stall_is_reported_once(cplx):
+    """qmcspl_slater_sync: ERR_TIMEOUT for the stalled launch, nothing before it and nothing after."""
+    from paper_1309_6250_gb300 import _lib
+    from paper_1309_6250_gb300.api import slater_kinetic, slater_sync
+    g = torch.Generator(device=dev()).manual_seed(9950)
+    val = torch.randn(2 * 9, 5, generator=g, device=dev(), dtype=torch.complex128 if cplx else torch.float64)
+    call = lambda: slater_kinetic(val, None, None, 2, 9, 5)
+    L = _lib.load()
+    try:
+        slater_sync()
+    except _lib.QmcsplError:
+        pass                                  # an earlier launch's
+    call()
+    slater_sync()
+    try:
+        L.qmcspl_debug_stall_slater(1)
+        out = call()
+        with pytest.raises(_lib.QmcsplError) as ei:
+            slater_sync()
+        assert ei.value.code == _lib.ERR_TIMEOUT
+    finally:
+        L.qmcspl_debug_stall_slater(0)
+    assert torch.isnan(out[0][0]) and not torch.isnan(out[0][1])
+    call()
+    slater_sync()
