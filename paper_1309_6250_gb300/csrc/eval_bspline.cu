@@ -524,6 +524,7 @@ template <> struct BspBlock<float, true> {
     static constexpr int large = QMCSPL_EVAL_THREADS_F32_LAP;
 };
 constexpr int kLargeLaunchRounds = 4;   // warp-task rounds from which the large shape is used
+inline bool large_launch(long long warps, int threads) { return warps >= (long long)kLargeLaunchRounds * sm_count() * (threads / 32); }
 
 template <typename T, bool LAPTAB, int THREADS, bool RAGGED, bool NOREC = false>
 __global__ void __launch_bounds__(THREADS, 1) bspline_vgl_kernel(const EvalArgs p)
@@ -765,8 +766,7 @@ int launch_typed(const EvalArgs& a, int threads, cudaStream_t st)
     if (small_launch(warps)) return launch_small<T, LAPTAB>(a, warps, st);
     constexpr int large = BspBlock<T, LAPTAB>::large;
     if constexpr (large != QMCSPL_EVAL_THREADS) {
-        if (warps >= (long long)kLargeLaunchRounds * sm_count() * (large / 32))
-            return launch_shape<T, LAPTAB, large>(a, warps, st);
+        if (large_launch(warps, large)) return launch_shape<T, LAPTAB, large>(a, warps, st);
     }
     return launch_shape<T, LAPTAB, QMCSPL_EVAL_THREADS>(a, warps, st);
 }
@@ -805,8 +805,11 @@ void set_outputs(const Handle* h, EvalArgs& a, void* val, void* grad, void* lap)
 // 32,768 positions x 16 orbitals, 48^3 26.8 -> 24.0 us (Hessian Laplacian 18.4 -> 14.4), 9,000 x 16 12.3 -> 10.2,
 // 12,000 x 128 47.2 -> 45.1, 24,000 x 64 47.5 -> 45.1, 24,000 x 128 bfloat16 61.0 -> 59.1.  The large shape has
 // no such form, and there the pass is the faster one: 30,000 x 128 102 us against 116, 30,000 x 64 58 against
-// 65.  So it is for several tiles of one or two lanes, which would each reduce all three axes: 12,000 x 109
-// bfloat16 37.1 us against 39.7, 40,000 x 40 62.7 against 62.6.
+// 65.  Tables without a large shape take the same line: near it both are alike, and over more rounds the
+// pass is the faster one for many lanes (Hessian Laplacian, 64^3 x 64 orbitals, 30,000 positions 46.1 us with the pass,
+// 45.0 without, 200,000 222 and 234; bfloat16, Laplacian table, 64^3 x 128, 30,000 116.5 and 119.3, 200,000 668 and
+// 708; few lanes the other way, 47.3 against 41.5 at 120,000 x 16).  So it is for several tiles of one or two lanes,
+// which would each reduce all three axes: 12,000 x 109 bfloat16 37.1 us against 39.7, 40,000 x 40 62.7 against 62.6.
 bool eval_shares_coordinates(const Handle* h, long long n_pos)
 {
     if (h->storage != QMCSPL_F32 && h->storage != QMCSPL_BF16) return false;
@@ -814,7 +817,7 @@ bool eval_shares_coordinates(const Handle* h, long long n_pos)
     if (h->bloch || h->block_threads == 640 || (h->lanes_log2 < 2 && h->tiles > 1)) return false;
     const int gpw = 32 >> h->lanes_log2;
     const long long warps = (n_pos * h->tiles + gpw - 1) / gpw;
-    return warps < (long long)kLargeLaunchRounds * sm_count() * (640 / 32);
+    return !large_launch(warps, BspBlock<float, true>::large);
 }
 
 int launch_bspline_vgl(const Handle* h, const double* pos, const Prepared& pr, long long n_pos, void* val,
@@ -847,7 +850,6 @@ int launch_batched(int n_cells, const Handle* const* hs, const double* const* po
     // QMCSPL_BATCH_AUTO: cells of at least kLargeLaunchRounds rounds of warp tasks (512-thread
     // blocks on every SM) get their own launch, the others share one batched launch;
     // QMCSPL_BATCH_SINGLE: every cell in the batched launch; QMCSPL_BATCH_SPLIT: every cell alone
-    const long long large = (long long)kLargeLaunchRounds * sm_count() * (QMCSPL_EVAL_THREADS / 32);
     int nb = 0;
     B.start[0] = 0;
     for (int c = 0; c < n_cells; ++c) {
@@ -861,7 +863,7 @@ int launch_batched(int n_cells, const Handle* const* hs, const double* const* po
         set_outputs(hs[c], a, val[c], grad[c], lap[c]);
         const int gpw = 32 >> a.lanes_log2;
         const long long warps = (a.n_pos * a.tiles + gpw - 1) / gpw;
-        const bool alone = launch == QMCSPL_BATCH_SPLIT || (launch == QMCSPL_BATCH_AUTO && warps >= large);
+        const bool alone = launch == QMCSPL_BATCH_SPLIT || (launch == QMCSPL_BATCH_AUTO && large_launch(warps, QMCSPL_EVAL_THREADS));
         if (alone) {
             if (warps == 0) continue;
             const int rc = launch_bspline_vgl(hs[c], pos[c], pr[c], n_pos[c], val[c], grad[c], lap[c], st);
