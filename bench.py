@@ -793,6 +793,28 @@ def bench_batched(args, dev, stream, l1=None):
     return res
 
 
+def kernel_launches(call):
+    """Kernels that one call launches, counted in a capture of it (never replayed)."""
+    import ctypes
+    import torch
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        call()
+    rt = ctypes.CDLL("libcudart.so.13")      # the runtime that torch and libqmcspl.so have loaded
+    graph, n, kind = ctypes.c_void_p(g.raw_cuda_graph()), ctypes.c_size_t(0), ctypes.c_int()
+    if rt.cudaGraphGetNodes(graph, None, ctypes.byref(n)):
+        raise RuntimeError("cudaGraphGetNodes failed")
+    nodes = (ctypes.c_void_p * n.value)()
+    if rt.cudaGraphGetNodes(graph, nodes, ctypes.byref(n)):
+        raise RuntimeError("cudaGraphGetNodes failed")
+    kernels = 0
+    for node in nodes:
+        if rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)):
+            raise RuntimeError("cudaGraphNodeGetType failed")
+        kernels += kind.value == 0           # cudaGraphNodeTypeKernel
+    return kernels
+
+
 def run_ours(args):
     import torch
     rank, ws, dist = dist_setup()
@@ -836,9 +858,7 @@ def run_ours(args):
     order_name = spl.resolved_order(n_pos)     # the library's rule (qmcspl_get_order)
     staged = order_name == "pencil"
     kernel_name = "bspline_vgl_staged_kernel" if staged else "bspline_vgl_kernel"
-    # sorted: records/bins, scan, place + evaluation; input order: a records pass from 8192
-    # positions on (Bloch handles: always, for the phases) + evaluation
-    kernels_per_step = 4 if order_name != "input" else (2 if n_pos >= 8192 or info["bloch"] else 1)
+    kernels_per_step = kernel_launches(eager)
 
     sampler = ClockSampler(dev.index if dev.index is not None else 0)
     for _ in range(args.warmup):
