@@ -12,6 +12,9 @@ host outputs back) every step.  The table (934 MB for FP32) and the outputs
 (1.34 GB) are both far larger than the 129 MB L2, so no extra flush is needed.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
+
+prints one JSON line on standard output; the secondary legs (other storage types and methods,
+batches, adjoints, Bloch orbitals, the Slater consumer) go to standard error as another.
 """
 from __future__ import annotations
 
@@ -793,6 +796,16 @@ def bench_batched(args, dev, stream, l1=None):
     return res
 
 
+# secondary legs of a run (17 KB beside the headline's 6: a reader of the line may cut it at 16)
+LEGS = ("variants", "batched", "methods_si8_48", "methods_mgo64_96", "backward_si64_72", "backward_mgo64_96",
+        "bloch_mgo64_96", "slater_consumer_mgo64", "general_degree_si8_48")
+
+
+def split_line(line):
+    """(the run's one line on standard output, its secondary legs as a line on standard error)"""
+    return {k: v for k, v in line.items() if k not in LEGS}, {"legs": {k: line[k] for k in LEGS if k in line}}
+
+
 def kernel_launches(call):
     """Kernels that one call launches, counted in a capture of it (never replayed)."""
     import ctypes
@@ -1072,6 +1085,8 @@ def run_ours(args):
         "general_degree_si8_48": general,
     }
     if rank == 0:
+        line, legs = split_line(line)
+        print(json.dumps(legs), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
     if dist:
         dist.barrier()
