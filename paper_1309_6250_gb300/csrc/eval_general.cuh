@@ -311,7 +311,11 @@ int launch_one(const EvalArgs& a, bool laptab, cudaStream_t st)
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kEvalThreads, 0);
     if (e != cudaSuccess) return cuda_error(e, "occupancy query");
-    if (per_sm < 1) per_sm = 1;
+    // Rows that are not whole 16-byte chunks, eight scalar stores per lane: once the coordinates come from
+    // records, the stores of a second block of the short uniform degree-1 kernel push the first one's half-filled
+    // sectors out (bfloat16, 64^3, 80,000 positions x 127 orbitals: 158 us with one block per SM, 203 with two; x 128,
+    // whole chunks, 115 and 88).  On graded grids, whose coordinates cost more, two are the faster (185 and 217).
+    if (per_sm < 1 || (DEG == 1 && !NONUNI && Traits<T>::E == 8 && a.rec && !a.vec_out)) per_sm = 1;
     const long long cap = (long long)sm_count() * per_sm;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
