@@ -520,14 +520,15 @@ int qmcspl_eval_vgl_noalloc(qmcspl_t h, const double* pos, long long n_pos, void
  *   drift  device double[n_walkers][n_elec][3] or NULL (needs grad); complex dtypes
  *          double[n_walkers][n_elec][3][2]
  *   stream cudaStream_t; asynchronous
- * The inversion is Gauss-Jordan elimination with row pivoting in shared memory, one thread
- * block per walker, in FP64 or in double-float (arith); complex entries are pivoted on the
- * largest modulus, and in double-float each of their parts is a float pair.  An exactly
+ * The inversion is Gauss-Jordan elimination with row pivoting in FP64 or in double-float (arith);
+ * complex entries are pivoted on the largest modulus, and in double-float each of their parts is a
+ * float pair.  Double-float blocks of up to 128 electrons (96 for complex dtypes) are kept in
+ * registers, a cluster of two thread blocks per walker; all others in shared memory, one thread block
+ * per walker.  The sums of kinetic energy and drift are FP64 in every kernel.  An exactly
  * singular block gives sign 0, logdet -inf and NaN kinetic energy and drift for that walker;
- * nearly singular blocks lose accuracy as the condition number grows.  In the double-float kernels
- * for up to 128 electrons per block (96 for complex dtypes) warps wait for one another's pivot
- * columns; should such a wait run out, every output of its walker is NaN, sign and logdet included,
- * and qmcspl_slater_sync reports it.
+ * nearly singular blocks lose accuracy as the condition number grows.  In the register kernels warps
+ * wait for one another's pivot columns; should such a wait run out, every output of its walker is NaN,
+ * sign and logdet included, and qmcspl_slater_sync reports it.
  */
 #define QMCSPL_SLATER_MAX_BLOCK 160
 #define QMCSPL_SLATER_MAX_COMPLEX_BLOCK 112

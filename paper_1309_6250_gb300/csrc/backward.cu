@@ -264,6 +264,9 @@ __device__ __forceinline__ void bwd_position(const BwdArgs& b, long long ip, boo
 
 // Blocks of four warps: the float kernels' 168 registers per thread let three of them (12 warps) run
 // on an SM, where one block of eight warps did (4,096 positions x 128 orbitals, both adjoints: 159 -> 148 us).
+// The other types have the registers for eight warps either way and gain where few warps are spread wider or end
+// more evenly (FP64, 10,000 x 16, both adjoints 472 -> 394 us); two sizes lose (FP64 10,000 x 128 2.57 -> 2.65 ms,
+// bfloat16 3,000 x 64, 64^3, 69 -> 76 us), and blocks of eight warps for large launches gave the gains back with them.
 constexpr int kBwdThreads = 128;
 template <typename T, bool LAPTAB, bool BLOCH, bool COEF>
 __global__ void __launch_bounds__(kBwdThreads, std::is_same<T, float>::value && !BLOCH ? 3 : 2) bspline_bwd_kernel(const BwdArgs b)

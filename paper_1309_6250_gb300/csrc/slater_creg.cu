@@ -7,11 +7,10 @@
 // packed FP32 operations per two entries: 64 x 64 blocks need 2,048 x 54 / 64 = 1,728 SM clocks per
 // elimination step.  slater_cdf_kernel, which it replaces here, moves 32 bytes of shared memory per
 // entry and step and meets at four barriers.  The final sums are FP64 here as there (two operations per
-// SM clock): in double-float they had 1.03 to 1.10 times
-// the drift's rms error, and neither a double's last bits nor its range.  Measured, 4,096 walkers x
-// (64 + 64), complex float orbitals 10.18 -> 5.24 ms (5.56 with double-float sums), complex double 9.57 -> 5.39;
-// 4,096 x (32 + 32) 3.49 -> 0.95 ms (0.92), 4,096 x (12 + 11) 1.35 -> 0.41 (0.40), 1,024 x (96 + 96)
-// 12.1 -> 5.39 (4.52).
+// SM clock): as double-float sums they had 1.03 to 1.10 times the drift's rms error and not the range of a
+// double.  Measured, 4,096 walkers x (64 + 64), complex float orbitals 10.18 -> 5.25 ms (5.56 with double-float
+// sums), complex double 9.57 -> 5.39; 4,096 x (32 + 32) 3.49 -> 0.95 ms (0.92), 4,096 x (12 + 11) 1.35 -> 0.41
+// (0.40), 1,024 x (96 + 96) 12.1 -> 5.42 (4.52).
 //
 // A lane keeps RL rows of CP column pairs, each as four packed pairs (re and im, high and low): 64
 // registers, 72 for 65 to 96 electrons.  97 to 112 electrons would need 98 of 128 and stay with

@@ -34,7 +34,8 @@
 //   the warp that holds column k + 1 brings that column up to date first, finds the next pivot (the
 //     largest |entry| over rows not yet used) and writes the column and 1 / pivot;
 //   every lane updates its entries.
-// The arithmetic of an entry is that of slater_df_kernel, operation for operation.
+// The updates are slater_df_kernel's error-free multiply-adds on the same operands; the renormalisation takes
+// three operations (quick_norm2) instead of a full two-sum, to the same result.
 // After n steps entry (i, j) is the inverse's row (step at which i was the pivot), column p_j.
 #include <cooperative_groups.h>
 
@@ -47,8 +48,8 @@ namespace cg = cooperative_groups;
 
 __device__ int timed_out;   // read and cleared by qmcspl_slater_sync
 
-// RL rows per lane, CP column pairs per lane, NW warps; `per_sm` CTAs of at most 128 registers per
-// thread fit on an SM.  G: spin blocks of at most 32 G electrons.
+// RL rows per lane, CP column pairs per lane, NW warps; `per_sm` CTAs fit on an SM with at most 85 registers
+// per thread for G = 1 (the compiler takes 80) and 128 for the others.  G: spin blocks of at most 32 G electrons.
 template <int G> struct RegShape;
 template <> struct RegShape<1> { static constexpr int RL = 1, CP = 8, NW = 2, per_sm = 12; };
 template <> struct RegShape<2> { static constexpr int RL = 2, CP = 8, NW = 4, per_sm = 4; };
